@@ -80,7 +80,7 @@ struct TcPlan {
     // shared-memory offsets; act holds slots x 2 buffers of act_bytes (row form: one buffer)
     uint32_t o_act, o_w0, o_w1, o_f32, o_rowtab, o_sitetab, o_spins, o_res, o_bar, o_extra, total;
     // row form (rows = 1, local energies): activations [kc][(xp * Lp + yp) * G + g][16 B] updated in place,
-    // rows_total rows per plane; a 4 KB zero block; the MMA lists; the layer images of layers >= 1 sit wimg
+    // rows_total rows per plane (wide form, rows = 2: the same without the padded columns, x in place of xp); a 4 KB zero block; the MMA lists; the layer images of layers >= 1 sit wimg
     // bytes after the tap-form images
     int rows, rows_total;
     uint32_t wimg, o_zero, o_mtab;
@@ -97,6 +97,9 @@ struct TcPlan {
 // are the same for every entry (SBO = 128 bytes, tcgen05 version bit).
 constexpr int kMtabLayer = 64, kMtab0 = 32;
 constexpr uint32_t kMtabBytes = 16u * kIssuers * (kMtabLayer + kMtab0) + 16u * kIssuers;   // + counts
+// zero block (A and B of the zeroing MMA): K chunks 2 KB apart, so 2 KB + 16 bytes per row of the larger operand
+// (128 rows; the wide form's B has up to 256)
+constexpr uint32_t kZeroRows = 4096, kZeroWide = 6144;
 
 __host__ __device__ inline uint32_t al16(uint32_t v) { return (v + 15u) & ~15u; }
 
@@ -668,19 +671,21 @@ __device__ void row_build_mtab(const TcPlan &pl, const TcShared &sh, int iw) {
 
 // Spins of the group to the layer-0 im2col: row x * 128 + m (m = y * G + g),
 // K0 columns tap-major (one-hot channel minor), as build_slot writes them.
-// Threads 0 .. 255 each keep one accumulator row m and walk every other
-// column x; the 3 x 3 neighbourhood comes from the row's three lattice rows.
+// Each group of 128 threads keeps one accumulator row m a thread and walks
+// its share of the columns x; the 3 x 3 neighbourhood comes from the row's
+// three lattice rows.
 __device__ void build_rows(const TcPlan &pl, const TcShared &sh) {
     const int G = pl.G, N = pl.N, L = pl.L;
     const uint32_t a0 = row_act(pl, sh);
     const uint32_t one = 0x3F80u, minus_one = 0xBF80u;   // bf16 +1, -1
-    if (threadIdx.x < 256) {
+    const int step = (int)(blockDim.x >> 7);
+    if ((int)threadIdx.x < 128 * step) {
         const int m = threadIdx.x & 127;
         const bool valid = m < G * L;
         const int y = valid ? m / G : 0, g = valid ? m - y * G : 0;
         const int8_t *sp = sh.spins + g * N;
         const int yr[3] = {(y == 0 ? L - 1 : y - 1) * L, y * L, (y == L - 1 ? 0 : y + 1) * L};
-        for (int x = (int)(threadIdx.x >> 7); x < L; x += 2) {
+        for (int x = (int)(threadIdx.x >> 7); x < L; x += step) {
             uint32_t w[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) w[i] = 0u;
@@ -990,9 +995,280 @@ __device__ bool row_forward(const TcPlan &pl, const TcShared &sh, const unsigned
     return true;
 }
 
+// ---------------------------------------------------------------- wide row form (32 channels, one block per SM)
+// The row form for accumulators too wide for two blocks (L * C up to all 512
+// tensor-memory columns). With one block per SM nothing else fills the tensor
+// core while this block's epilogue runs, so the two overlap inside the block:
+// the output columns are split into halves A = [0, H) and B = [H, L), each
+// issued by its own warp and completed by its own commit, and the epilogue
+// warps take a layer's columns in three stages:
+//   0  columns 1 .. H - 2, once A has completed: B reads only the input columns
+//      H - 1 .. L - 1 and 0, so these may be overwritten while B still runs;
+//   1  columns 0, H - 1, H, L - 1, once B has completed: with them the next
+//      layer's A has its whole input (columns L - 1, 0 .. H) and may start;
+//   2  columns H + 1 .. L - 2, written while the next layer's A runs; then the
+//      next layer's B may start.
+// The activations are still updated in place (one buffer), the warps meet at
+// mbarriers (bar_tile[0, 1]: A, B done; bar_tile[2, 3]: stages 1, 2 written)
+// instead of block barriers, and every output keeps the tap form's order
+// (dy, dx, K halves), so the results are bitwise those of the tap form.
+// Bound: the operand path of the N = 3C MMAs (7 KB per MMA of 128 x 96 x 16,
+// 56 cycles, against 120 for the tap form's three N = 32 MMAs).
+constexpr int kWideEpi = 16;
+constexpr int kWideThreads = 32 * (kWideEpi + kIssuers);
+
+// Issuer iw's MMA lists (half A or B), as row_build_mtab's without padded
+// columns: the input column x is read at plane row x Lp G.
+template <int C>
+__device__ void wide_build_mtab(const TcPlan &pl, const TcShared &sh, int iw) {
+    uint4 *tab = reinterpret_cast<uint4 *>(sh.base + pl.o_mtab) + iw * (kMtabLayer + kMtab0);
+    int *cnt = reinterpret_cast<int *>(sh.base + pl.o_mtab + 16u * kIssuers * (kMtabLayer + kMtab0)) + 2 * iw;
+    const uint32_t act = row_act(pl, sh);
+    const int L = pl.L, H = L / 2, xa = iw == 0 ? 0 : H, xb = iw == 0 ? H : L;
+    constexpr int KC = C / 8;
+    int n = 0;
+    for (int dy = 0; dy < 3; ++dy)
+        for (int xi = xa - 1; xi <= xb; ++xi) {
+            const int lo = max(xi - 1, xa), hi = min(xi + 1, xb - 1), j0 = lo - (xi - 1);
+            const int xs = xi < 0 ? L - 1 : (xi == L ? 0 : xi);
+            const uint32_t arow = (uint32_t)((xs * pl.Lp + dy) * pl.G);
+            for (int kk = 0; kk < C / 16; ++kk)
+                tab[n++] = make_uint4(desc_lo(act + arow * 16u + (uint32_t)(2 * kk) * pl.plane, pl.plane),
+                                      desc_lo((uint32_t)(((dy * KC + 2 * kk) * 3 * C + j0 * C) * 16), 3 * C * 16),
+                                      (uint32_t)(lo * C), ptx::idesc_bf16(128, (hi - lo + 1) * C));
+        }
+    cnt[0] = n;
+    int n0 = 0;
+    for (int x = xa; x < xb; ++x)
+        for (int kk = 0; kk < pl.K0 / 16; ++kk)
+            tab[kMtabLayer + n0++] = make_uint4(desc_lo(act + (uint32_t)x * 128u * 16u + (uint32_t)(2 * kk) * pl.plane,
+                                                        pl.plane),
+                                                desc_lo((uint32_t)(2 * kk * C * 16), C * 16),
+                                                (uint32_t)(x * C) | (kk ? 0x80000000u : 0u), ptx::idesc_bf16(128, C));
+    cnt[1] = n0;
+}
+
+// Issue layer l's MMAs of half iw (the whole issuer warp) and commit them to
+// bar_tile[iw]. False if the wait for the weights gave up.
+template <int C>
+__device__ bool wide_issue(const TcPlan &pl, const TcShared &sh, const unsigned char *packed, const TcState &st, int l,
+                           int iw) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t q = st.wseq + (uint32_t)l;
+    if (!__all_sync(0xffffffffu, wait_or_abort(&sh.bar_w[q & 1], (q >> 1) & 1, sh.abort_flag))) return false;
+    ptx::tc_fence_after();
+    const uint32_t tmem = *sh.tmem_addr;
+    const uint4 *tab = reinterpret_cast<const uint4 *>(sh.base + pl.o_mtab) + iw * (kMtabLayer + kMtab0);
+    const int *cnt = reinterpret_cast<const int *>(sh.base + pl.o_mtab + 16u * kIssuers * (kMtabLayer + kMtab0)) + 2 * iw;
+    const uint32_t wlo = ptx::smem_u32(sh.base + ((q & 1) ? pl.o_w1 : pl.o_w0)) >> 4;
+    constexpr uint64_t hi = (uint64_t)kDescHi << 32;
+    if (l == 0) {
+        const int n0 = cnt[1];
+        for (int k = 0; k < n0; ++k) {
+            const uint4 e = tab[kMtabLayer + k];
+            ptx::mma_bf16_elect(tmem + (e.z & 0x7FFFFFFFu), hi | e.x, hi | (e.y + wlo), e.w, e.z >> 31);
+        }
+    } else {
+        const int H = pl.L / 2, xa = iw == 0 ? 0 : H, xb = iw == 0 ? H : pl.L;
+        const uint64_t z = hi | desc_lo(ptx::smem_u32(sh.base + pl.o_zero), 2048);
+        ptx::mma_bf16_elect(tmem + (uint32_t)(xa * C), z, z, ptx::idesc_bf16(128, (xb - xa) * C), 0u);
+        const int n = cnt[0];
+#pragma unroll 4
+        for (int k = 0; k < n; ++k) {
+            const uint4 e = tab[k];
+            ptx::mma_bf16_elect(tmem + e.z, hi | e.x, hi | (e.y + wlo), e.w, 1u);
+        }
+    }
+    ptx::mma_commit_elect(&sh.bar_tile[iw]);
+    // the next layer's weights into the other buffer: its last readers, layer l - 1's MMAs of both halves, had
+    // completed before stage 1 of that layer was written (or before the block barrier between groups)
+    if (lane == 0 && iw == 0) issue_weight_load(pl, sh, packed, q + 1, st.wbase);
+    return true;
+}
+
+// Columns of epilogue stage s: their number and the i-th one.
+__device__ __forceinline__ int wide_stage_cols(int L, int s) {
+    return s == 0 ? L / 2 - 2 : (s == 1 ? 4 : L - L / 2 - 2);
+}
+__device__ __forceinline__ int wide_stage_col(int L, int s, int i) {
+    const int H = L / 2;
+    if (s == 0) return 1 + i;
+    if (s == 2) return H + 1 + i;
+    return i < 2 ? (i == 0 ? 0 : H - 1) : (i == 2 ? H : L - 1);
+}
+
+// Where the head contributions of column x start (floats): in the column's
+// own activation rows, so that stage 0 may write them while half B still
+// reads the others, skewed by x words against bank conflicts in the head.
+__device__ __forceinline__ int wide_contrib(const TcPlan &pl, int x) { return x * (pl.Lp * pl.G * 4 + 1); }
+
+// Epilogue of layer l (epilogue warps): a warp takes a TMEM lane quarter and,
+// of the columns of each stage, its share of (column, 16 channels) units; after
+// the last layer whole columns, whose contributions sum the channels in order.
+template <int C>
+__device__ bool wide_epilogue(const TcPlan &pl, const TcShared &sh, uint32_t &ph, int l, int *err) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = warp & 3;
+    const bool last = l == pl.n_layers - 1;
+    const int G = pl.G, L = pl.L, Lp = pl.Lp;
+    constexpr int NH = C / 16;
+    const int h = warp >> 2, nh = pl.epi >> 2;
+    const int half = h % NH, cg = last ? h : h / NH, ncg = last ? nh : nh / NH;
+    const float *bias = sh.f32 + l * C;
+    const float *wa = sh.f32 + pl.n_layers * C;
+    const uint32_t act = row_act(pl, sh);
+    float *contrib = reinterpret_cast<float *>(sh.base + pl.o_act);
+    const int m = quarter * 32 + lane;
+    const bool valid = m < G * L;
+    const int y = valid ? m / G : 0, g = valid ? m - y * G : 0;
+    const int yimg = y == 0 ? L + 1 : (y == L - 1 ? 0 : -1);
+    const uint32_t amain = act + (uint32_t)((y + 1) * G + g) * 16u + (uint32_t)(2 * half) * pl.plane;
+    const int dimg = (yimg - (y + 1)) * G * 16;
+    const uint32_t tmem = *sh.tmem_addr + ((uint32_t)(quarter * 32) << 16);
+    float hb[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) hb[c] = 0.5f * bias[16 * half + c];
+    for (int s = 0; s < 3; ++s) {
+        if (s < 2) {
+            if (!__all_sync(0xffffffffu, wait_sleep_or_abort(&sh.bar_tile[s], (ph >> s) & 1u, sh.abort_flag)))
+                return false;
+            ph ^= 1u << s;
+            ptx::tc_fence_after();
+        }
+        const int n = wide_stage_cols(L, s);
+        if (!last) {
+            uint32_t ra[16], rb[16];
+            if (cg < n) {
+                ptx::tmem_ld16_nowait(tmem + (uint32_t)(wide_stage_col(L, s, cg) * C + 16 * half), ra);
+                ptx::tmem_wait_ld();
+                ptx::reg_fence16(ra);
+            }
+            for (int i = cg; i < n; i += ncg) {
+                const int x = wide_stage_col(L, s, i);
+                const bool more = i + ncg < n;
+                if (more) ptx::tmem_ld16_nowait(tmem + (uint32_t)(wide_stage_col(L, s, i + ncg) * C + 16 * half), rb);
+                uint32_t w[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const float2 o = ptx::silu_bias2(make_float2(__uint_as_float(ra[2 * c]), __uint_as_float(ra[2 * c + 1])),
+                                                     make_float2(hb[2 * c], hb[2 * c + 1]));
+                    w[c] = ptx::pack_bf16(o.x, o.y);
+                }
+                if (valid && NQS_INDEX_OK((x * Lp + y + 1) * G + g < pl.rows_total &&
+                                              (yimg < 0 || (x * Lp + yimg) * G + g < pl.rows_total), err)) {
+                    const uint32_t a = amain + (uint32_t)(x * Lp * G) * 16u;
+                    ptx::st_shared_v4(a, w[0], w[1], w[2], w[3]);
+                    ptx::st_shared_v4(a + pl.plane, w[4], w[5], w[6], w[7]);
+                    if (yimg >= 0) {
+                        ptx::st_shared_v4(a + (uint32_t)dimg, w[0], w[1], w[2], w[3]);
+                        ptx::st_shared_v4(a + (uint32_t)dimg + pl.plane, w[4], w[5], w[6], w[7]);
+                    }
+                }
+                if (more) {
+                    ptx::tmem_wait_ld();
+                    ptx::reg_fence16(rb);
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) ra[c] = rb[c];
+                }
+            }
+            if (s > 0) {   // this warp's columns of the stage are drained and written
+                ptx::tc_fence_before();
+                ptx::fence_async_smem();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(&sh.bar_tile[1 + s]);
+            }
+        } else {
+            for (int i = cg; i < n; i += ncg) {
+                const int x = wide_stage_col(L, s, i);
+                uint32_t r[NH][16];
+#pragma unroll
+                for (int q = 0; q < NH; ++q) ptx::tmem_ld16_nowait(tmem + (uint32_t)(x * C + 16 * q), r[q]);
+                ptx::tmem_wait_ld();
+#pragma unroll
+                for (int q = 0; q < NH; ++q) ptx::reg_fence16(r[q]);
+                if (!valid) continue;
+                float ca = 0.f, cp = 0.f;
+#pragma unroll
+                for (int c4 = 0; c4 < C; c4 += 4) {
+                    const float4 b = *reinterpret_cast<const float4 *>(bias + c4);
+                    const float4 xa = *reinterpret_cast<const float4 *>(wa + c4);
+                    const float4 xq = *reinterpret_cast<const float4 *>(wa + C + c4);
+                    const uint32_t *v = r[c4 >> 4];
+                    const int k0 = c4 & 15;
+                    const float2 h01 = ptx::silu_fast2(make_float2(__uint_as_float(v[k0]), __uint_as_float(v[k0 + 1])),
+                                                       make_float2(b.x, b.y));
+                    const float2 h23 = ptx::silu_fast2(make_float2(__uint_as_float(v[k0 + 2]), __uint_as_float(v[k0 + 3])),
+                                                       make_float2(b.z, b.w));
+                    ca = fmaf(xa.x, h01.x, ca), cp = fmaf(xq.x, h01.x, cp);
+                    ca = fmaf(xa.y, h01.y, ca), cp = fmaf(xq.y, h01.y, cp);
+                    ca = fmaf(xa.z, h23.x, ca), cp = fmaf(xq.z, h23.x, cp);
+                    ca = fmaf(xa.w, h23.y, ca), cp = fmaf(xq.w, h23.y, cp);
+                }
+                const int idx = wide_contrib(pl, x) + y * G + g;
+                contrib[idx] = ca;
+                contrib[idx + L * G] = cp;
+            }
+        }
+    }
+    return true;
+}
+
+// Sums of the head contributions per configuration, in head_slot's order
+// (lane k takes sites k, k + 32, ..., then the xor-shuffle tree); one warp per
+// configuration and output.
+__device__ void wide_head(const TcPlan &pl, const TcShared &sh) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = pl.G, L = pl.L;
+    const float *contrib = reinterpret_cast<const float *>(sh.base + pl.o_act);
+    for (int t = warp; t < 2 * G; t += (int)(blockDim.x >> 5)) {
+        const int g = t >> 1, o = t & 1;
+        float sum = 0.f;
+        for (int site = lane; site < pl.N; site += 32) {
+            const int y = site / L, x = site - y * L;
+            sum += contrib[wide_contrib(pl, x) + o * L * G + y * G + g];
+        }
+#pragma unroll
+        for (int k = 16; k > 0; k >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, k);
+        if (lane == 0) sh.res[o * G + g] = (double)sum;
+    }
+    __syncthreads();
+}
+
+// Evaluate the group's G configurations (sh.spins) in the wide row form;
+// results in sh.res. False if a wait gave up (the block must stop).
+template <int C>
+__device__ bool wide_forward(const TcPlan &pl, const TcShared &sh, const unsigned char *packed, TcState &st, int *err) {
+    build_rows(pl, sh);
+    const int warp = threadIdx.x >> 5, nl = pl.n_layers;
+    uint32_t ph = st.tphase;
+    bool ok = true;
+    if (warp >= pl.epi) {
+        const int iw = warp - pl.epi;
+        for (int l = 0; ok && l < nl; ++l) {
+            if (l > 0) {   // stage 1 + iw of the layer before: this half's input is written, its accumulators drained
+                ok = __all_sync(0xffffffffu, wait_or_abort(&sh.bar_tile[2 + iw], (ph >> (2 + iw)) & 1u, sh.abort_flag));
+                ph ^= 4u << iw;
+            }
+            ok = ok && wide_issue<C>(pl, sh, packed, st, l, iw);
+        }
+    } else {
+        for (int l = 0; ok && l < nl; ++l) ok = wide_epilogue<C>(pl, sh, ph, l, err);
+    }
+    if (!ok) raise_abort(sh, err);
+    // every thread leaves with the same barrier phases: A and B complete nl times, the stages nl - 1 times
+    st.tphase ^= (nl & 1) ? 3u : 12u;
+    st.wissued = st.wseq + (uint32_t)nl + 1u;
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    if (*(volatile int *)sh.abort_flag) return false;
+    wide_head(pl, sh);
+    st.wseq += (uint32_t)nl;
+    return true;
+}
+
 // ---------------------------------------------------------------- kernel prologue / epilogue
-// Once per block: barriers (fixed offset 0), tensor memory.
-__device__ void tc_init(TcShared &sh, unsigned char *smem, uint32_t tmem_cols, TcState &st) {
+// Once per block: barriers (fixed offset 0), tensor memory. stage_arrivals:
+// arrivals that complete a phase of bar_tile[2, 3] (the wide form's stages).
+__device__ void tc_init(TcShared &sh, unsigned char *smem, uint32_t tmem_cols, TcState &st, uint32_t stage_arrivals = 1) {
     sh.base = smem;
     sh.bar_w = reinterpret_cast<uint64_t *>(smem);
     sh.bar_tile = sh.bar_w + 2;
@@ -1001,7 +1277,8 @@ __device__ void tc_init(TcShared &sh, unsigned char *smem, uint32_t tmem_cols, T
     if (threadIdx.x == 0) {
         ptx::mbar_init(&sh.bar_w[0], 1);
         ptx::mbar_init(&sh.bar_w[1], 1);
-        for (int t = 0; t < kMaxSlots * kMaxTiles; ++t) ptx::mbar_init(&sh.bar_tile[t], 1);
+        for (int t = 0; t < kMaxSlots * kMaxTiles; ++t)
+            ptx::mbar_init(&sh.bar_tile[t], (t == 2 || t == 3) ? stage_arrivals : 1u);
         *sh.abort_flag = 0;
         ptx::fence_mbar_init();
     }
@@ -1062,32 +1339,28 @@ __device__ void tc_bind(const TcPlan &pl, TcShared &sh, const unsigned char *pac
     st.wissued += 1;
 }
 
-// Bind the block to a row-form plan: parameters, site and neighbour tables,
+// Bind the block to a row-form plan (either form): parameters, MMA lists,
 // zeroed activations and zero block, first weight load.
 __device__ void row_bind(const TcPlan &pl, TcShared &sh, const unsigned char *packed, TcState &st) {
     unsigned char *smem = sh.base;
     sh.spins = reinterpret_cast<int8_t *>(smem + pl.o_spins);
     sh.rowtab = nullptr;
-    sh.sitetab = reinterpret_cast<const uint2 *>(smem + pl.o_sitetab);
+    sh.sitetab = nullptr;
     sh.f32 = reinterpret_cast<float *>(smem + pl.o_f32);
     sh.res = reinterpret_cast<double *>(smem + pl.o_res);
     const float *src = reinterpret_cast<const float *>(packed);
     for (uint32_t i = threadIdx.x; i < pl.f32_count; i += blockDim.x) sh.f32[i] = src[i];
-    uint2 *sitetab = reinterpret_cast<uint2 *>(smem + pl.o_sitetab);
-    for (int s = threadIdx.x; s < pl.N; s += blockDim.x) {
-        int pos[4];
-        const int n = images(pl.L, pl.Lp, s % pl.L, s / pl.L, pos);
-        sitetab[s] = pack4(pos, n);
-    }
     // zero the activations (rows no output writes are read only by discarded
     // accumulator rows, but stay finite) and the zero block
     for (uint32_t i = threadIdx.x; i < pl.act_bytes / 4; i += blockDim.x)
         reinterpret_cast<uint32_t *>(smem + pl.o_act)[i] = 0u;
-    for (uint32_t i = threadIdx.x; i < 4096 / 4; i += blockDim.x) reinterpret_cast<uint32_t *>(smem + pl.o_zero)[i] = 0u;
+    const uint32_t zero = pl.rows == 2 ? kZeroWide : kZeroRows;
+    for (uint32_t i = threadIdx.x; i < zero / 4; i += blockDim.x) reinterpret_cast<uint32_t *>(smem + pl.o_zero)[i] = 0u;
     {
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, iw = warp - pl.epi;
         if (lane == 0 && iw >= 0 && iw < kIssuers) {
-            if (pl.C == 16) row_build_mtab<16>(pl, sh, iw);
+            if (pl.rows == 2) wide_build_mtab<32>(pl, sh, iw);
+            else if (pl.C == 16) row_build_mtab<16>(pl, sh, iw);
             else row_build_mtab<32>(pl, sh, iw);
         }
     }
@@ -1175,8 +1448,9 @@ __global__ void __launch_bounds__(kTcThreads, kMinBlocks<C>) logpsi_tc_kernel(Tc
 // configurations, evaluate sigma and all of them in groups, then
 // E_loc = H_diag + sum_k H_k exp((a'_k - a) + i (phi'_k - phi)) in float64,
 // every term of the sample at once, fixed-order block reduction.
-// ROWS: the configurations go through the row form (no cones).
-template <int C, bool ROWS = false, bool F8 = false>
+// FORM: the forward the configurations go through (0 tap form, with cones if
+// there is a cache; 1 row form, 2 wide row form, both dense).
+template <int C, int FORM = 0, bool F8 = false>
 __device__ bool eloc_sample(const TcPlan &pl, const Problem &p, const TcShared &sh, TcState &st,
                             const unsigned char *packed, const int8_t *cfg, const double *logpsi_s, double *out_s,
                             int *err, unsigned char *cache) {
@@ -1190,14 +1464,15 @@ __device__ bool eloc_sample(const TcPlan &pl, const Problem &p, const TcShared &
     EnumScratch *scr = reinterpret_cast<EnumScratch *>(ex + al16(N) + al16(4 * chunk) + al16(8 * chunk) +
                                                        al16(4 * (N + 1)));
     double *ref = reinterpret_cast<double *>(scr + 1);   // a0, phi0
-    double *lp = ref + 4;                                 // [chunk + 1][2]: (a, phi) of every list entry
-    double *fsum = lp + 2 * (chunk + 1);                  // [258] fixed-order sum scratch
+    float *lp = reinterpret_cast<float *>(ref + 4);       // [chunk + 1][2]: (a, phi) of every list entry (the head's
+                                                          // float32 sums, so the float keeps every bit)
+    double *fsum = ref + 4 + (chunk + 1);                 // [258] fixed-order sum scratch
     int16_t *ord = reinterpret_cast<int16_t *>(fsum + 258);   // [chunk] evaluation order of the entries
     int *roll = reinterpret_cast<int *>(ord + ((chunk + 1) & ~1));   // [32] per configuration of a group
     const int recompute = logpsi_s == nullptr;
     // the cone of every connected configuration is evaluated alone when the
     // sample itself is evaluated here (its activations fill the cache)
-    const bool cone = !ROWS && cache != nullptr && recompute && pl.slots == 1;
+    const bool cone = FORM == 0 && cache != nullptr && recompute && pl.slots == 1;
     for (int r = threadIdx.x; r < N; r += blockDim.x) sigma[r] = cfg[r];
     __syncthreads();
     if (p.model == NQS_MODEL_TJ) snake_prefix(p, sigma, cum, *scr);
@@ -1278,7 +1553,9 @@ __device__ bool eloc_sample(const TcPlan &pl, const Problem &p, const TcShared &
                 }
             }
             __syncthreads();
-            if (ROWS) {
+            if constexpr (FORM == 2) {
+                if (!wide_forward<C>(pl, sh, packed, st, err)) return false;
+            } else if constexpr (FORM == 1) {
                 if (!row_forward<C, F8>(pl, sh, packed, st, err)) return false;
             } else if (!tc_forward<C>(pl, sh, packed, st, err, band, cache, (cone && lead && e0 == 0) ? cache : nullptr)) {
                 return false;
@@ -1287,8 +1564,8 @@ __device__ bool eloc_sample(const TcPlan &pl, const Problem &p, const TcShared &
                 const int c = threadIdx.x, sl = c / G, g = c - sl * G;
                 const int q = e0 + c - lead;
                 const int idx = q < 0 ? 0 : ord[q] + lead;
-                lp[2 * idx] = sh.res[sl * 2 * G + g];
-                lp[2 * idx + 1] = sh.res[sl * 2 * G + G + g];
+                lp[2 * idx] = (float)sh.res[sl * 2 * G + g];
+                lp[2 * idx + 1] = (float)sh.res[sl * 2 * G + G + g];
             }
             __syncthreads();
         }
@@ -1297,9 +1574,9 @@ __device__ bool eloc_sample(const TcPlan &pl, const Problem &p, const TcShared &
         __syncthreads();
         // off-diagonal terms in an order independent of the block size
         const double2 tsum = fixed_order_sum2(nconn, [&](int k) {
-            const double m = ch[k] * exp(lp[2 * (k + lead)] - ref[0]);
+            const double m = ch[k] * exp((double)lp[2 * (k + lead)] - ref[0]);
             double sn, cs;
-            sincos(lp[2 * (k + lead) + 1] - ref[1], &sn, &cs);
+            sincos((double)lp[2 * (k + lead) + 1] - ref[1], &sn, &cs);
             return make_double2(m * cs, m * sn);
         }, fsum);
         sr_tot += tsum.x;
@@ -1343,8 +1620,25 @@ __global__ void __launch_bounds__(kTcThreads, 2)
     tc_init(sh, smem, pl.tmem_cols, st);
     row_bind(pl, sh, packed, st);
     for (int64_t s = blockIdx.x; s < n; s += gridDim.x)
-        if (!eloc_sample<C, true, F8>(pl, p, sh, st, packed, configs + s * p.N, logpsi ? logpsi + 2 * s : nullptr,
+        if (!eloc_sample<C, 1, F8>(pl, p, sh, st, packed, configs + s * p.N, logpsi ? logpsi + 2 * s : nullptr,
                                       out + 2 * s, err, nullptr))
+            break;
+    tc_teardown(pl, sh, st);
+}
+
+// Local energies through the wide row form (32 channels, one block per SM).
+template <int C>
+__global__ void __launch_bounds__(kWideThreads, 1)
+    eloc_wide_kernel(TcPlan pl, Problem p, const unsigned char *packed, const int8_t *configs, const double *logpsi,
+                     int64_t n, double *out, int *err) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    TcShared sh;
+    TcState st;
+    tc_init(sh, smem, pl.tmem_cols, st, (uint32_t)pl.epi);
+    row_bind(pl, sh, packed, st);
+    for (int64_t s = blockIdx.x; s < n; s += gridDim.x)
+        if (!eloc_sample<C, 2>(pl, p, sh, st, packed, configs + s * p.N, logpsi ? logpsi + 2 * s : nullptr, out + 2 * s,
+                               err, nullptr))
             break;
     tc_teardown(pl, sh, st);
 }
@@ -1709,7 +2003,7 @@ bool make_row_plan(const Problem &p, size_t max_smem, int extra_bytes, TcPlan *o
     uint32_t o = kBarBytes;
     pl.o_bar = 0;
     pl.o_act = o; o = al16(o + pl.act_bytes);
-    pl.o_zero = o; o = al16(o + 4096);
+    pl.o_zero = o; o = al16(o + kZeroRows);
     pl.o_w0 = o; o = al16(o + pl.wbytes);
     pl.o_w1 = o; o = al16(o + pl.wbytes);
     pl.o_f32 = o; o = al16(o + pl.f32_count * 4);
@@ -1730,6 +2024,56 @@ bool make_row_plan(const Problem &p, size_t max_smem, int extra_bytes, TcPlan *o
     return true;
 }
 
+// Wide row-form plan (32 channels): G = min(16, 128 / L) configurations per
+// block, one block per SM, up to all 512 accumulator columns.
+bool make_wide_plan(const Problem &p, size_t max_smem, int extra_bytes, TcPlan *out, std::string *why, int G = 0) {
+    if (p.C != 32 || p.L * p.C > 512) { *why = "wide row form: 32 channels, L * C <= 512"; return false; }
+    TcPlan pl{};
+    pl.rows = 2;
+    pl.ctas = 1;
+    pl.epi = kWideEpi;
+    pl.L = p.L;
+    pl.Lp = p.L + 2;
+    pl.N = p.N;
+    pl.G = G > 0 ? std::min(std::min(G, 16), 128 / p.L) : std::min(16, 128 / p.L);
+    pl.C = p.C;
+    pl.KC = p.C / 8;
+    pl.c_in = p.c_in;
+    pl.n_layers = p.n_layers;
+    pl.slots = 1;
+    plan_weights(p, pl);
+    pl.wimg = (uint32_t)(p.n_layers - 1) * pl.wbytes;
+    pl.n_tiles = 1;
+    // activations x Lp G + yp G + g; the last A operand starts 2 G rows into column L - 1 and spans 128 rows; the
+    // im2col of layer 0 takes L x 128
+    pl.rows_total = std::max(p.L * pl.Lp * pl.G + 128 - p.L * pl.G, p.L * 128);
+    pl.rows_total = (pl.rows_total + 7) & ~7;
+    pl.rbuf = pl.rows_total;
+    pl.plane = (uint32_t)pl.rows_total * 16u;
+    pl.act_bytes = pl.plane * (uint32_t)pl.KC;
+    pl.slot_cols = (uint32_t)(p.L * p.C);
+    uint32_t cols = 32;
+    while (cols < pl.slot_cols) cols <<= 1;
+    pl.tmem_cols = cols;
+    uint32_t o = kBarBytes;
+    pl.o_bar = 0;
+    pl.o_act = o; o = al16(o + pl.act_bytes);
+    pl.o_zero = o; o = al16(o + kZeroWide);
+    pl.o_w0 = o; o = al16(o + pl.wbytes);
+    pl.o_w1 = o; o = al16(o + pl.wbytes);
+    pl.o_f32 = o; o = al16(o + pl.f32_count * 4);
+    pl.o_mtab = o; o = al16(o + kMtabBytes);
+    pl.o_spins = o; o = al16(o + pl.G * p.N);
+    pl.o_res = o; o = al16(o + 16 * pl.G);
+    pl.o_extra = o; o = al16(o + extra_bytes);
+    const uint32_t sm_bytes = 233472u;   // 228 KB per SM, 1 KB reserved per block
+    while (cols * (sm_bytes / (o + 1024u)) > 512u || 2u * (o + 1024u) <= sm_bytes) o += 1024u;   // one block per SM
+    pl.total = o;
+    if (pl.total > max_smem) { *why = "wide row form: shared memory plan exceeds the per-block limit"; return false; }
+    *out = pl;
+    return true;
+}
+
 // Whether the local-energy launch uses the row form (NQS_TC_ROWS=0 turns it
 // off, NQS_TC_ROWS=G forces G configurations per group: tuning and A/B
 // comparisons).
@@ -1741,7 +2085,8 @@ bool use_row_form(const Problem &p, size_t max_smem, TcPlan *out) {
         if (G == 0) return false;
     }
     std::string why;
-    return make_row_plan(p, max_smem, eloc_extra(p), out, &why, G);
+    return make_row_plan(p, max_smem, eloc_extra(p), out, &why, G) ||
+           make_wide_plan(p, max_smem, eloc_extra(p), out, &why, G);
 }
 
 bool make_plan(const Problem &p, int G, int slots, int ctas, size_t max_smem, int extra_bytes, TcPlan *out,
@@ -1799,7 +2144,7 @@ bool make_plan(const Problem &p, int G, int slots, int ctas, size_t max_smem, in
 int eloc_extra(const Problem &p) {
     const int chunk = bond_chunk(p);
     return (int)(al16(p.N) + al16(4 * chunk) + al16(8 * chunk) + al16(4 * (p.N + 1)) + sizeof(EnumScratch) +
-                 4 * sizeof(double) + 16 * (chunk + 1) + 8 * 258 + 2 * ((chunk + 1) & ~1) + 4 * 32);
+                 4 * sizeof(double) + 8 * (chunk + 1) + 8 * 258 + 2 * ((chunk + 1) & ~1) + 4 * 32);
 }
 
 int sample_extra(const Problem &p, int G, int slots) {
@@ -1976,6 +2321,13 @@ int launch_eloc_tc(const Problem &p, const double *, const void *packed, const i
     }
     if (use_row_form(p, env.max_smem, &pl)) {
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)env.num_sms * pl.ctas));
+        if (pl.rows == 2) {
+            auto k = eloc_wide_kernel<32>;
+            if (int rc = prep(k, pl, env)) return rc;
+            k<<<grid, 32 * (pl.epi + kIssuers), pl.total, env.stream>>>(pl, p, (const unsigned char *)packed, configs,
+                                                                        logpsi, n, out, env.err);
+            return check(env, "eloc_wide_kernel");
+        }
         NQS_TC_DISPATCH(p.C, {
             auto k = eloc_rows_kernel<CC>;
             if (int rc = prep(k, pl, env)) return rc;
@@ -2151,7 +2503,7 @@ int tc_describe_plan(const Problem &p, int kind, int64_t n, size_t max_smem, int
     out[5] = (int32_t)pl.total;
     out[6] = (int32_t)pl.tmem_cols;
     out[7] = (int32_t)grid;
-    out[8] = pl.rows;
+    out[8] = pl.rows != 0;
     return NQS_OK;
 }
 
