@@ -83,7 +83,7 @@ struct TcPlan {
     // rows_total rows per plane (wide form, rows = 2: the same without the padded columns, x in place of xp); a 4 KB zero block; the MMA lists; the layer images of layers >= 1 sit wimg
     // bytes after the tap-form images
     int rows, rows_total;
-    uint32_t wimg, o_zero, o_mtab;
+    uint32_t wimg, o_zero, o_mtab, o_lane;
     // weight loads of layers >= 1: bytes per layer (their stride in the packed image); f8: the row form with
     // e4m3 operands in layers >= 1 (f8bytes per layer image)
     uint32_t wstride, f8bytes;
@@ -219,6 +219,17 @@ __device__ __forceinline__ bool wait_sleep_or_abort(uint64_t *bar, uint32_t pari
         if (ptx::mbar_try_wait_sleep(bar, parity, 20000u)) return true;
         if (*(volatile const int *)abort_flag) return false;
         if (ptx::globaltimer_ns() - t0 > ptx::kSleepWaitLimitNs) return false;
+    }
+    return false;
+}
+
+// The wide form's wait: tight polling in rounds of 64, the abort flag read
+// between rounds. Gives up when another thread raised it or after the
+// iteration limit.
+__device__ __forceinline__ bool wide_wait(uint64_t *bar, uint32_t parity, const int *abort_flag) {
+    for (long long it = 0; it < ptx::kWaitLimit; it += 64) {
+        if (ptx::mbar_poll(bar, parity, 64u)) return true;
+        if (*(volatile const int *)abort_flag) return false;
     }
     return false;
 }
@@ -671,21 +682,19 @@ __device__ void row_build_mtab(const TcPlan &pl, const TcShared &sh, int iw) {
 
 // Spins of the group to the layer-0 im2col: row x * 128 + m (m = y * G + g),
 // K0 columns tap-major (one-hot channel minor), as build_slot writes them.
-// Each group of 128 threads keeps one accumulator row m a thread and walks
-// its share of the columns x; the 3 x 3 neighbourhood comes from the row's
-// three lattice rows.
+// Threads 0 .. 255 each keep one accumulator row m and walk every other
+// column x; the 3 x 3 neighbourhood comes from the row's three lattice rows.
 __device__ void build_rows(const TcPlan &pl, const TcShared &sh) {
     const int G = pl.G, N = pl.N, L = pl.L;
     const uint32_t a0 = row_act(pl, sh);
     const uint32_t one = 0x3F80u, minus_one = 0xBF80u;   // bf16 +1, -1
-    const int step = (int)(blockDim.x >> 7);
-    if ((int)threadIdx.x < 128 * step) {
+    if (threadIdx.x < 256) {
         const int m = threadIdx.x & 127;
         const bool valid = m < G * L;
         const int y = valid ? m / G : 0, g = valid ? m - y * G : 0;
         const int8_t *sp = sh.spins + g * N;
         const int yr[3] = {(y == 0 ? L - 1 : y - 1) * L, y * L, (y == L - 1 ? 0 : y + 1) * L};
-        for (int x = (int)(threadIdx.x >> 7); x < L; x += step) {
+        for (int x = (int)(threadIdx.x >> 7); x < L; x += 2) {
             uint32_t w[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) w[i] = 0u;
@@ -995,106 +1004,308 @@ __device__ bool row_forward(const TcPlan &pl, const TcShared &sh, const unsigned
     return true;
 }
 
-// ---------------------------------------------------------------- wide row form (32 channels, one block per SM)
-// The row form for accumulators too wide for two blocks (L * C up to all 512
-// tensor-memory columns). With one block per SM nothing else fills the tensor
-// core while this block's epilogue runs, so the two overlap inside the block:
-// the output columns are split into halves A = [0, H) and B = [H, L), each
-// issued by its own warp and completed by its own commit, and the epilogue
-// warps take a layer's columns in three stages:
-//   0  columns 1 .. H - 2, once A has completed: B reads only the input columns
-//      H - 1 .. L - 1 and 0, so these may be overwritten while B still runs;
+// ---------------------------------------------------------------- wide row form
+// The row form with the MMAs and the epilogue of a layer overlapped inside the
+// block and connected configurations restricted to their cones.
+//
+// Overlap. The output columns are split into halves A = [0, H) and B = [H, L),
+// each issued by its own warp and completed by its own commit, and the
+// epilogue warps take a layer's columns in three stages:
+//   0  A's columns that B does not read, once A has completed: B reads the
+//      input columns H - 1 .. L - 1 and 0, so columns 1 .. H - 2 may be
+//      overwritten while B still runs;
 //   1  columns 0, H - 1, H, L - 1, once B has completed: with them the next
 //      layer's A has its whole input (columns L - 1, 0 .. H) and may start;
 //   2  columns H + 1 .. L - 2, written while the next layer's A runs; then the
 //      next layer's B may start.
 // The activations are still updated in place (one buffer), the warps meet at
 // mbarriers (bar_tile[0, 1]: A, B done; bar_tile[2, 3]: stages 1, 2 written)
-// instead of block barriers, and every output keeps the tap form's order
-// (dy, dx, K halves), so the results are bitwise those of the tap form.
-// Bound: the operand path of the N = 3C MMAs (7 KB per MMA of 128 x 96 x 16,
-// 56 cycles, against 120 for the tap form's three N = 32 MMAs).
-constexpr int kWideEpi = 16;
-constexpr int kWideThreads = 32 * (kWideEpi + kIssuers);
+// instead of block barriers.
+//
+// Cones. A connected configuration differs from its sample in two sites of
+// one column (class 0) or of two adjacent columns (class 1). Each
+// configuration of a group is rolled along x so that its pair sits at column
+// H - 1 (and H); layer l then computes columns H - 2 - l .. H + cls + l only
+// (wide_cols), and of the columns outside it those that the next layer reads are
+// copied (cp.async, with their y images; two warps of their own) from a
+// per-block cache of the sample's own activations, rolled by the same amount:
+// those left of H after A, the others after B. The group that holds the sample is evaluated
+// densely and writes the cache. The last layer is dense.
+//
+// Every output keeps the tap form's order (dy, dx, K halves), so the results
+// are bitwise those of the tap form. Bound: the shared-memory operand path of
+// the N = 3C MMAs (128 x 96 x 16: 7 KB, 56 cycles, against 120 for the tap
+// form's three N = 32 MMAs), the epilogue's stores, which share it, and the
+// latency of the stages. Measured (GB300): J1-J2 16x16, 32 channels, 8 layers,
+// 4,096 samples 127.2 ms in the tap form, 75.2 dense and 67.9 with cones here;
+// t-J 12x12, 32 channels, 6 layers, 2,048 samples 10.97 -> 7.41; J1-J2 10x10,
+// 16 channels, 6 layers, 8,192 samples 12.27 in the row form -> 11.04.
+constexpr int kWideEpi = 16;    // epilogue warps with one block per SM (two blocks: kMaxEpiWarps each)
+// warps that copy the columns outside a band while the epilogue warps work (launches with cones only; they fit beside
+// the issuers in the register allocation's granule of four warps)
+constexpr int kWideFill = 2;
+template <int C> constexpr int kWideBlocks = C == 16 ? 2 : 1;
+template <int C> constexpr int kWideThreads = 32 * (C == 16 ? kMaxEpiWarps + kIssuers : kWideEpi + kIssuers + kWideFill);
 
-// Issuer iw's MMA lists (half A or B), as row_build_mtab's without padded
-// columns: the input column x is read at plane row x Lp G.
-template <int C>
-__device__ void wide_build_mtab(const TcPlan &pl, const TcShared &sh, int iw) {
-    uint4 *tab = reinterpret_cast<uint4 *>(sh.base + pl.o_mtab) + iw * (kMtabLayer + kMtab0);
-    int *cnt = reinterpret_cast<int *>(sh.base + pl.o_mtab + 16u * kIssuers * (kMtabLayer + kMtab0)) + 2 * iw;
-    const uint32_t act = row_act(pl, sh);
-    const int L = pl.L, H = L / 2, xa = iw == 0 ? 0 : H, xb = iw == 0 ? H : L;
-    constexpr int KC = C / 8;
-    int n = 0;
-    for (int dy = 0; dy < 3; ++dy)
-        for (int xi = xa - 1; xi <= xb; ++xi) {
-            const int lo = max(xi - 1, xa), hi = min(xi + 1, xb - 1), j0 = lo - (xi - 1);
-            const int xs = xi < 0 ? L - 1 : (xi == L ? 0 : xi);
-            const uint32_t arow = (uint32_t)((xs * pl.Lp + dy) * pl.G);
-            for (int kk = 0; kk < C / 16; ++kk)
-                tab[n++] = make_uint4(desc_lo(act + arow * 16u + (uint32_t)(2 * kk) * pl.plane, pl.plane),
-                                      desc_lo((uint32_t)(((dy * KC + 2 * kk) * 3 * C + j0 * C) * 16), 3 * C * 16),
-                                      (uint32_t)(lo * C), ptx::idesc_bf16(128, (hi - lo + 1) * C));
-        }
-    cnt[0] = n;
-    int n0 = 0;
-    for (int x = xa; x < xb; ++x)
-        for (int kk = 0; kk < pl.K0 / 16; ++kk)
-            tab[kMtabLayer + n0++] = make_uint4(desc_lo(act + (uint32_t)x * 128u * 16u + (uint32_t)(2 * kk) * pl.plane,
-                                                        pl.plane),
-                                                desc_lo((uint32_t)(2 * kk * C * 16), C * 16),
-                                                (uint32_t)(x * C) | (kk ? 0x80000000u : 0u), ptx::idesc_bf16(128, C));
-    cnt[1] = n0;
+// Columns [lo, hi] that layer l computes for a group of class cls (< 0: every
+// column of every layer); false if it computes all of them. (A band never
+// reaches column L - 1: it would be as wide as the lattice.)
+__device__ __forceinline__ bool wide_cols(const TcPlan &pl, int cls, int l, int &lo, int &hi) {
+    const int H = pl.L / 2;
+    lo = H - 2 - l;
+    hi = H + cls + l;
+    if (cls >= 0 && l < pl.n_layers - 1 && lo >= 0 && hi < pl.L && hi - lo + 1 < pl.L) return true;
+    lo = 0;
+    hi = pl.L - 1;
+    return false;
 }
 
-// Issue layer l's MMAs of half iw (the whole issuer warp) and commit them to
-// bar_tile[iw]. False if the wait for the weights gave up.
+// Per-block cache of the sample's activations of layers 0 .. n_layers - 2:
+// [layer][x][y][C / 8][16 bytes].
+__host__ __device__ inline size_t wide_cache_bytes(const TcPlan &pl) {
+    const size_t b = (size_t)(pl.n_layers - 1) * pl.N * pl.C * 2;
+    return (b + 255) & ~(size_t)255;
+}
+
+// Issue layer l's MMAs of half iw (one elected lane of the issuer warp) and
+// commit them to bar_tile[iw]. Layer 0: the im2col rows x * 128, one
+// N = C MMA per column and K half. Later layers, onto zeroed accumulators: per
+// kernel row dy and input column xi the outputs xi - 1 .. xi + 1 of the half, K
+// halves innermost. Broadcast values and the split into edge and interior
+// columns keep the descriptors in uniform registers with two additions an
+// interior MMA, so that one thread issues as fast as the operand path takes
+// them (45 cycles at N = 48, 54 at N = 96 on an idle SM; 66 and 57 with the
+// columns in one loop; the election in every MMA cost 8 - 17 % of the whole
+// kernel). False if the wait for the weights gave up.
 template <int C>
 __device__ bool wide_issue(const TcPlan &pl, const TcShared &sh, const unsigned char *packed, const TcState &st, int l,
-                           int iw) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t q = st.wseq + (uint32_t)l;
-    if (!__all_sync(0xffffffffu, wait_or_abort(&sh.bar_w[q & 1], (q >> 1) & 1, sh.abort_flag))) return false;
+                           int iw, int cls) {
+    const uint32_t q = __shfl_sync(0xffffffffu, st.wseq + (uint32_t)l, 0);
+    if (!__all_sync(0xffffffffu, wide_wait(&sh.bar_w[q & 1], (q >> 1) & 1, sh.abort_flag))) return false;
     ptx::tc_fence_after();
-    const uint32_t tmem = *sh.tmem_addr;
-    const uint4 *tab = reinterpret_cast<const uint4 *>(sh.base + pl.o_mtab) + iw * (kMtabLayer + kMtab0);
-    const int *cnt = reinterpret_cast<const int *>(sh.base + pl.o_mtab + 16u * kIssuers * (kMtabLayer + kMtab0)) + 2 * iw;
-    const uint32_t wlo = ptx::smem_u32(sh.base + ((q & 1) ? pl.o_w1 : pl.o_w0)) >> 4;
-    constexpr uint64_t hi = (uint64_t)kDescHi << 32;
-    if (l == 0) {
-        const int n0 = cnt[1];
-        for (int k = 0; k < n0; ++k) {
-            const uint4 e = tab[kMtabLayer + k];
-            ptx::mma_bf16_elect(tmem + (e.z & 0x7FFFFFFFu), hi | e.x, hi | (e.y + wlo), e.w, e.z >> 31);
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *sh.tmem_addr, 0);
+    const uint32_t wb = ptx::smem_u32(sh.base + ((q & 1) ? pl.o_w1 : pl.o_w0));
+    const uint32_t abase = desc_lo(row_act(pl, sh), pl.plane), kplane = pl.plane >> 3;   // two planes, 16-byte units
+    constexpr uint64_t dh = (uint64_t)kDescHi << 32;
+    constexpr int KC = C / 8;
+    constexpr uint32_t i1 = ptx::idesc_bf16(128, C), i2 = ptx::idesc_bf16(128, 2 * C), i3 = ptx::idesc_bf16(128, 3 * C);
+    int lo, hi;
+    wide_cols(pl, cls, l, lo, hi);
+    const int L = pl.L, H = L / 2, xa = iw == 0 ? lo : H, xb = iw == 0 ? H : hi + 1;
+    if (ptx::elect_one()) {
+        if (l == 0) {
+            const uint32_t bbase = desc_lo(wb, C * 16);
+            uint32_t a = abase + (uint32_t)(xa * 128), d = tmem + (uint32_t)(xa * C);
+            for (int x = xa; x < xb; ++x, a += 128u, d += C)
+                for (int kk = 0; kk < pl.K0 / 16; ++kk)
+                    ptx::mma_bf16(d, dh | (a + kk * kplane), dh | (bbase + (uint32_t)(2 * kk * C)), i1, kk ? 1u : 0u);
+        } else {
+            const uint64_t z = dh | desc_lo(ptx::smem_u32(sh.base + pl.o_zero), 2048);
+            ptx::mma_bf16(tmem + (uint32_t)(xa * C), z, z, ptx::idesc_bf16(128, (xb - xa) * C), 0u);
+            const uint32_t bbase = desc_lo(wb, 3 * C * 16), step = (uint32_t)(pl.Lp * pl.G);
+            const uint32_t left = (uint32_t)(xa == 0 ? L - 1 : xa - 1) * step, right = (uint32_t)(xb == L ? 0 : xb) * step;
+            const uint32_t dl = tmem + (uint32_t)(xa * C), dr = tmem + (uint32_t)((xb - 1) * C);
+            auto one = [&](uint32_t a, uint32_t b, uint32_t d, uint32_t idesc) {
+#pragma unroll
+                for (int kk = 0; kk < C / 16; ++kk)
+                    ptx::mma_bf16(d, dh | (a + kk * kplane), dh | (b + (uint32_t)(2 * kk * 3 * C)), idesc, 1u);
+            };
+            for (int dy = 0; dy < 3; ++dy) {
+                const uint32_t b = bbase + (uint32_t)(dy * KC * 3 * C), arow = abase + (uint32_t)(dy * pl.G);
+                uint32_t a = arow + (uint32_t)xa * step, d = dl;
+                one(arow + left, b + 2 * C, dl, i1);
+                if (xb - xa == 1) {
+                    one(a, b + C, dl, i1);
+                } else {
+                    one(a, b + C, dl, i2);
+#pragma unroll 2
+                    for (int xi = xa + 1; xi < xb - 1; ++xi, d += C) {
+                        a += step;
+                        one(a, b, d, i3);
+                    }
+                    one(a + step, b, d, i2);
+                }
+                one(arow + right, b, dr, i1);
+            }
         }
-    } else {
-        const int H = pl.L / 2, xa = iw == 0 ? 0 : H, xb = iw == 0 ? H : pl.L;
-        const uint64_t z = hi | desc_lo(ptx::smem_u32(sh.base + pl.o_zero), 2048);
-        ptx::mma_bf16_elect(tmem + (uint32_t)(xa * C), z, z, ptx::idesc_bf16(128, (xb - xa) * C), 0u);
-        const int n = cnt[0];
-#pragma unroll 4
-        for (int k = 0; k < n; ++k) {
-            const uint4 e = tab[k];
-            ptx::mma_bf16_elect(tmem + e.z, hi | e.x, hi | (e.y + wlo), e.w, 1u);
-        }
+        ptx::mma_commit(&sh.bar_tile[iw]);
+        // the next layer's weights into the other buffer: its last readers, layer l - 1's MMAs of both halves, had
+        // completed before stage 1 of that layer was written (or before the block barrier between groups)
+        if (iw == 0) issue_weight_load(pl, sh, packed, q + 1, st.wbase);
     }
-    ptx::mma_commit_elect(&sh.bar_tile[iw]);
-    // the next layer's weights into the other buffer: its last readers, layer l - 1's MMAs of both halves, had
-    // completed before stage 1 of that layer was written (or before the block barrier between groups)
-    if (lane == 0 && iw == 0) issue_weight_load(pl, sh, packed, q + 1, st.wbase);
+    __syncwarp();
     return true;
 }
 
-// Columns of epilogue stage s: their number and the i-th one.
-__device__ __forceinline__ int wide_stage_cols(int L, int s) {
-    return s == 0 ? L / 2 - 2 : (s == 1 ? 4 : L - L / 2 - 2);
+// What a thread knows about its accumulator row m = y G + g, from a table in
+// shared memory (built once per block: the divisions cost more than the load).
+struct WideRow {
+    int y, g;
+    bool valid;
+    uint32_t main;   // bytes from a column's first row to padded row y + 1 of configuration g
+    int dimg;        // from there to its periodic image along y (0: none)
+};
+
+__device__ __forceinline__ WideRow wide_row(const TcPlan &pl, const TcShared &sh, int m) {
+    const int4 e = reinterpret_cast<const int4 *>(sh.base + pl.o_lane)[m];
+    WideRow r;
+    r.y = e.x & 0xFF;
+    r.g = (e.x >> 8) & 0xFF;
+    r.valid = (e.x >> 16) != 0;
+    r.main = (uint32_t)e.y;
+    r.dimg = e.z;
+    return r;
 }
-__device__ __forceinline__ int wide_stage_col(int L, int s, int i) {
-    const int H = L / 2;
-    if (s == 0) return 1 + i;
-    if (s == 2) return H + 1 + i;
-    return i < 2 ? (i == 0 ? 0 : H - 1) : (i == 2 ? H : L - 1);
+
+// One configuration of the group: sigma with sites i and j exchanged (-1: as
+// it is), rolled along x: its column c is sigma's column c + roll.
+struct WideCfg {
+    int16_t i, j, roll, pad;
+};
+
+// Layer-0 im2col of columns lo .. hi: row x * 128 + m (m = y * G + g), K0
+// columns tap-major (one-hot channel minor), straight from the sample with
+// each row's exchange and roll applied. A group of 128 threads walks its share
+// of the columns with the 3 x 3 window in registers (three loads a column).
+__device__ void wide_build(const TcPlan &pl, const TcShared &sh, const int8_t *sigma, const WideCfg *cfgs, int lo,
+                           int hi) {
+    const int L = pl.L, groups = (int)(blockDim.x >> 7), grp = (int)(threadIdx.x >> 7), n = hi - lo + 1;
+    const int xb = lo + grp * n / groups, xe = grp < groups ? lo + (grp + 1) * n / groups : xb;
+    const int m = threadIdx.x & 127;
+    const WideRow w = wide_row(pl, sh, m);
+    if (xb < xe && w.valid) {
+        const WideCfg cf = cfgs[w.g];
+        const int i = cf.i, j = cf.j;
+        const int r0 = (w.y == 0 ? L - 1 : w.y - 1) * L, r1 = w.y * L, r2 = (w.y == L - 1 ? 0 : w.y + 1) * L;
+        auto at = [&](int site) -> uint32_t {   // the site's value after the exchange, as an unsigned byte
+            const int s = site == i ? j : (site == j ? i : site);
+            return reinterpret_cast<const uint8_t *>(sigma)[s];
+        };
+        const uint32_t a0 = row_act(pl, sh) + (uint32_t)m * 16u;
+        int x = xb - 1 + cf.roll;   // sigma's column of the window's next column
+        if (x < 0) x += L;
+        if (x >= L) x -= L;
+        if (pl.c_in == 1) {
+            // bf16 +-1: 0x3F80 with the byte's sign bit
+            auto enc = [&](int site) { return 0x3F80u | ((at(site) << 8) & 0x8000u); };
+            uint32_t p0 = 0, p1 = 0, p2 = 0, c0 = 0, c1 = 0, c2 = 0;
+            for (int k = xb - 1; k <= xe; ++k) {
+                const uint32_t n0 = enc(r0 + x), n1 = enc(r1 + x), n2 = enc(r2 + x);
+                x = x + 1 == L ? 0 : x + 1;
+                if (k > xb) {
+                    const uint32_t a = a0 + (uint32_t)(k - 1) * 2048u;
+                    ptx::st_shared_v4(a, p0 | (c0 << 16), n0 | (p1 << 16), c1 | (n1 << 16), p2 | (c2 << 16));
+                    ptx::st_shared_v4(a + pl.plane, n2, 0u, 0u, 0u);
+                }
+                p0 = c0, p1 = c1, p2 = c2;
+                c0 = n0, c1 = n1, c2 = n2;
+            }
+        } else {
+            // one-hot (hole, up, down) per tap: u = hole | up << 16, d = down
+            uint32_t u[9], d[9];
+#pragma unroll
+            for (int o = 0; o < 9; ++o) u[o] = d[o] = 0u;
+            for (int k = xb - 1; k <= xe; ++k) {
+#pragma unroll
+                for (int o = 0; o < 9; o += 3) {
+                    u[o] = u[o + 1], u[o + 1] = u[o + 2];
+                    d[o] = d[o + 1], d[o + 1] = d[o + 2];
+                    const uint32_t v = at((o == 0 ? r0 : (o == 3 ? r1 : r2)) + x);
+                    u[o + 2] = v == 0u ? 0x3F80u : (v == 1u ? 0x3F800000u : 0u);
+                    d[o + 2] = v == 255u ? 0x3F80u : 0u;
+                }
+                x = x + 1 == L ? 0 : x + 1;
+                if (k > xb) {
+                    uint32_t q[16];
+#pragma unroll
+                    for (int o = 0; o < 8; o += 2) {   // two taps: h u | d h | u d
+                        q[3 * (o / 2)] = u[o];
+                        q[3 * (o / 2) + 1] = d[o] | (u[o + 1] << 16);
+                        q[3 * (o / 2) + 2] = (u[o + 1] >> 16) | (d[o + 1] << 16);
+                    }
+                    q[12] = u[8];
+                    q[13] = d[8];
+                    q[14] = q[15] = 0u;
+                    const uint32_t a = a0 + (uint32_t)(k - 1) * 2048u;
+#pragma unroll
+                    for (int kc = 0; kc < 4; ++kc)
+                        ptx::st_shared_v4(a + (uint32_t)kc * pl.plane, q[4 * kc], q[4 * kc + 1], q[4 * kc + 2],
+                                          q[4 * kc + 3]);
+                }
+            }
+        }
+    }
+    ptx::fence_async_smem();
+    __syncthreads();
+}
+
+// Columns the next layer reads that layer l, banded, does not compute: left of
+// the band in part 0, right of it in part 1. Returns false if the next layer's
+// half A reads column L - 1 (part 1 must then be in place before it starts).
+__device__ __forceinline__ bool wide_outside(const TcPlan &pl, int cls, int l, int part, int &c0, int &c1) {
+    int lo, hi, nlo, nhi;
+    wide_cols(pl, cls, l, lo, hi);
+    const bool next = wide_cols(pl, cls, l + 1, nlo, nhi);
+    const bool wraps = !next || nlo == 0;
+    c0 = part == 0 ? (wraps ? 0 : nlo - 1) : hi + 1;
+    c1 = part == 0 ? lo - 1 : (wraps ? pl.L - 1 : nhi + 1);
+    return !wraps;
+}
+
+// Copy the columns [c0, c1] of layer l's activations, every padded row and
+// configuration, from the sample's cache (fill warp w; asynchronous). Lanes: planes fastest, so that a quarter warp reads whole
+// position records (C * 2 bytes each); the plane stride (make_wide_plan)
+// spreads its writes over the banks.
+template <int C>
+__device__ __forceinline__ void wide_fill(const TcPlan &pl, const TcShared &sh, const WideCfg *cfgs, int l, int c0, int c1,
+                                          const unsigned char *cache, int w) {
+    constexpr int KC = C / 8;
+    const int lane = threadIdx.x & 31, G = pl.G, L = pl.L, Lp = pl.Lp;
+    const unsigned char *src = cache + (size_t)l * pl.N * KC * 16;
+    const uint32_t act = row_act(pl, sh);
+    for (int e = lane; e < KC * G; e += 32) {
+        const int kc = e & (KC - 1), g = e / KC;
+        const uint32_t dst = act + (uint32_t)kc * pl.plane + (uint32_t)g * 16u;
+        int x = c0 + cfgs[g].roll;
+        if (x >= L) x -= L;
+        for (int c = c0; c <= c1; ++c) {
+            const unsigned char *col = src + (x * L * KC + kc) * 16;
+            const uint32_t dc = dst + (uint32_t)(c * Lp * G) * 16u;
+            for (int yp = w; yp < Lp; yp += kWideFill) {
+                const int y = yp == 0 ? L - 1 : (yp == Lp - 1 ? 0 : yp - 1);
+                ptx::cp_async16(dc + (uint32_t)(yp * G) * 16u, col + y * KC * 16);
+            }
+            x = x + 1 == L ? 0 : x + 1;
+        }
+    }
+}
+
+// The fill warps' share of a banded layer l: part 0 once half A's MMAs have
+// completed (no MMA then reads those columns), part 1 once B's have; each
+// arrives with the epilogue warps' stages 1 and 2.
+template <int C>
+__device__ bool wide_fill_layer(const TcPlan &pl, const TcShared &sh, uint32_t &ph, int l, int cls, const WideCfg *cfgs,
+                                const unsigned char *cache, int w) {
+    int lo, hi, c0, c1;
+    const bool banded = wide_cols(pl, cls, l, lo, hi);
+    bool apart = true;
+    for (int s = 0; s < 2; ++s) {
+        if (!__all_sync(0xffffffffu, wide_wait(&sh.bar_tile[s], (ph >> s) & 1u, sh.abort_flag))) return false;
+        ph ^= 1u << s;
+        if (banded) {
+            apart = wide_outside(pl, cls, l, s, c0, c1);
+            wide_fill<C>(pl, sh, cfgs, l, c0, c1, cache, w);
+            ptx::cp_async_commit();
+        }
+    }
+    for (int s = 1; s < 3 && l < pl.n_layers - 1; ++s) {
+        if (s == 1 && apart) ptx::cp_async_wait_group<1>();
+        else ptx::cp_async_wait_group<0>();
+        ptx::fence_async_smem();
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(&sh.bar_tile[1 + s]);
+    }
+    return true;
 }
 
 // Where the head contributions of column x start (floats): in the column's
@@ -1105,70 +1316,78 @@ __device__ __forceinline__ int wide_contrib(const TcPlan &pl, int x) { return x 
 // Epilogue of layer l (epilogue warps): a warp takes a TMEM lane quarter and,
 // of the columns of each stage, its share of (column, 16 channels) units; after
 // the last layer whole columns, whose contributions sum the channels in order.
+// cache_w: where the group that holds the sample as configuration 0 stores its
+// activations (or null).
 template <int C>
-__device__ bool wide_epilogue(const TcPlan &pl, const TcShared &sh, uint32_t &ph, int l, int *err) {
+__device__ bool wide_epilogue(const TcPlan &pl, const TcShared &sh, const WideRow &w, uint32_t &ph, int l, int *err,
+                              int cls, unsigned char *cache_w) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = warp & 3;
     const bool last = l == pl.n_layers - 1;
-    const int G = pl.G, L = pl.L, Lp = pl.Lp;
+    const int L = pl.L, H = L / 2;
     constexpr int NH = C / 16;
     const int h = warp >> 2, nh = pl.epi >> 2;
     const int half = h % NH, cg = last ? h : h / NH, ncg = last ? nh : nh / NH;
-    const float *bias = sh.f32 + l * C;
+    const float *bias = sh.f32 + l * C;   // halved
     const float *wa = sh.f32 + pl.n_layers * C;
     const uint32_t act = row_act(pl, sh);
     float *contrib = reinterpret_cast<float *>(sh.base + pl.o_act);
-    const int m = quarter * 32 + lane;
-    const bool valid = m < G * L;
-    const int y = valid ? m / G : 0, g = valid ? m - y * G : 0;
-    const int yimg = y == 0 ? L + 1 : (y == L - 1 ? 0 : -1);
-    const uint32_t amain = act + (uint32_t)((y + 1) * G + g) * 16u + (uint32_t)(2 * half) * pl.plane;
-    const int dimg = (yimg - (y + 1)) * G * 16;
-    const uint32_t tmem = *sh.tmem_addr + ((uint32_t)(quarter * 32) << 16);
-    float hb[16];
+    const uint32_t amain = act + w.main + (uint32_t)(2 * half) * pl.plane, colbytes = (uint32_t)(pl.Lp * pl.G) * 16u;
+    const uint32_t tmem = *sh.tmem_addr + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(last ? 0 : 16 * half);
+    unsigned char *cw = cache_w && w.valid && w.g == 0
+                            ? cache_w + ((size_t)(l * pl.N + w.y) * NH + half) * 32 : nullptr;   // + x L NH 32
+    int lo, hi;
+    const bool banded = wide_cols(pl, cls, l, lo, hi);
+    alignas(16) float hb[16];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) hb[c] = 0.5f * bias[16 * half + c];
+    for (int c = 0; c < 4; ++c)
+        *reinterpret_cast<float4 *>(hb + 4 * c) = *reinterpret_cast<const float4 *>(bias + 16 * half + 4 * c);
+    auto unit = [&](int x, const uint32_t (&r)[16]) {
+        uint32_t o[8];
+        ptx::silu_bias16(r, hb, o);
+        const uint32_t a = amain + (uint32_t)x * colbytes;
+        if (w.valid && NQS_INDEX_OK(a + pl.plane + 16u <= act + (uint32_t)(2 * half + 2) * pl.plane, err)) {
+            ptx::st_shared_v4(a, o[0], o[1], o[2], o[3]);
+            ptx::st_shared_v4(a + pl.plane, o[4], o[5], o[6], o[7]);
+            if (w.dimg) {
+                ptx::st_shared_v4(a + (uint32_t)w.dimg, o[0], o[1], o[2], o[3]);
+                ptx::st_shared_v4(a + (uint32_t)w.dimg + pl.plane, o[4], o[5], o[6], o[7]);
+            }
+            if (cw) {
+                uint4 *c4 = reinterpret_cast<uint4 *>(cw + (size_t)(x * L) * NH * 32);
+                c4[0] = make_uint4(o[0], o[1], o[2], o[3]);
+                c4[1] = make_uint4(o[4], o[5], o[6], o[7]);
+            }
+        }
+    };
+#pragma unroll 1
     for (int s = 0; s < 3; ++s) {
         if (s < 2) {
-            if (!__all_sync(0xffffffffu, wait_sleep_or_abort(&sh.bar_tile[s], (ph >> s) & 1u, sh.abort_flag)))
+            if (!__all_sync(0xffffffffu, wide_wait(&sh.bar_tile[s], (ph >> s) & 1u, sh.abort_flag)))
                 return false;
             ph ^= 1u << s;
             ptx::tc_fence_after();
         }
-        const int n = wide_stage_cols(L, s);
+        // the stage's columns: the i-th is first + i, or in a dense layer's stage 1 column 0, H - 1, H, L - 1
+        const int first = s == 0 ? (banded ? lo : 1) : (s == 1 ? H - 1 : H + 1);
+        const int n = s == 0 ? H - 1 - first : (s == 1 ? (banded ? 2 : 4) : (banded ? hi : L - 2) - H);
+        const bool ends = s == 1 && !banded;
+        auto col = [&](int i) { return ends ? (i == 0 ? 0 : (i == 3 ? L - 1 : H - 2 + i)) : first + i; };
         if (!last) {
             uint32_t ra[16], rb[16];
-            if (cg < n) {
-                ptx::tmem_ld16_nowait(tmem + (uint32_t)(wide_stage_col(L, s, cg) * C + 16 * half), ra);
+            int i = cg;
+            if (i < n) ptx::tmem_ld16_nowait(tmem + (uint32_t)(col(i) * C), ra);
+            while (i < n) {   // the next unit's accumulators load while this one is processed
                 ptx::tmem_wait_ld();
                 ptx::reg_fence16(ra);
-            }
-            for (int i = cg; i < n; i += ncg) {
-                const int x = wide_stage_col(L, s, i);
-                const bool more = i + ncg < n;
-                if (more) ptx::tmem_ld16_nowait(tmem + (uint32_t)(wide_stage_col(L, s, i + ncg) * C + 16 * half), rb);
-                uint32_t w[8];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const float2 o = ptx::silu_bias2(make_float2(__uint_as_float(ra[2 * c]), __uint_as_float(ra[2 * c + 1])),
-                                                     make_float2(hb[2 * c], hb[2 * c + 1]));
-                    w[c] = ptx::pack_bf16(o.x, o.y);
-                }
-                if (valid && NQS_INDEX_OK((x * Lp + y + 1) * G + g < pl.rows_total &&
-                                              (yimg < 0 || (x * Lp + yimg) * G + g < pl.rows_total), err)) {
-                    const uint32_t a = amain + (uint32_t)(x * Lp * G) * 16u;
-                    ptx::st_shared_v4(a, w[0], w[1], w[2], w[3]);
-                    ptx::st_shared_v4(a + pl.plane, w[4], w[5], w[6], w[7]);
-                    if (yimg >= 0) {
-                        ptx::st_shared_v4(a + (uint32_t)dimg, w[0], w[1], w[2], w[3]);
-                        ptx::st_shared_v4(a + (uint32_t)dimg + pl.plane, w[4], w[5], w[6], w[7]);
-                    }
-                }
-                if (more) {
-                    ptx::tmem_wait_ld();
-                    ptx::reg_fence16(rb);
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) ra[c] = rb[c];
-                }
+                if (i + ncg < n) ptx::tmem_ld16_nowait(tmem + (uint32_t)(col(i + ncg) * C), rb);
+                unit(col(i), ra);
+                i += ncg;
+                if (i >= n) break;
+                ptx::tmem_wait_ld();
+                ptx::reg_fence16(rb);
+                if (i + ncg < n) ptx::tmem_ld16_nowait(tmem + (uint32_t)(col(i + ncg) * C), ra);
+                unit(col(i), rb);
+                i += ncg;
             }
             if (s > 0) {   // this warp's columns of the stage are drained and written
                 ptx::tc_fence_before();
@@ -1178,14 +1397,14 @@ __device__ bool wide_epilogue(const TcPlan &pl, const TcShared &sh, uint32_t &ph
             }
         } else {
             for (int i = cg; i < n; i += ncg) {
-                const int x = wide_stage_col(L, s, i);
+                const int x = col(i);
                 uint32_t r[NH][16];
 #pragma unroll
                 for (int q = 0; q < NH; ++q) ptx::tmem_ld16_nowait(tmem + (uint32_t)(x * C + 16 * q), r[q]);
                 ptx::tmem_wait_ld();
 #pragma unroll
                 for (int q = 0; q < NH; ++q) ptx::reg_fence16(r[q]);
-                if (!valid) continue;
+                if (!w.valid) continue;
                 float ca = 0.f, cp = 0.f;
 #pragma unroll
                 for (int c4 = 0; c4 < C; c4 += 4) {
@@ -1194,18 +1413,18 @@ __device__ bool wide_epilogue(const TcPlan &pl, const TcShared &sh, uint32_t &ph
                     const float4 xq = *reinterpret_cast<const float4 *>(wa + C + c4);
                     const uint32_t *v = r[c4 >> 4];
                     const int k0 = c4 & 15;
-                    const float2 h01 = ptx::silu_fast2(make_float2(__uint_as_float(v[k0]), __uint_as_float(v[k0 + 1])),
+                    const float2 h01 = ptx::silu_bias2(make_float2(__uint_as_float(v[k0]), __uint_as_float(v[k0 + 1])),
                                                        make_float2(b.x, b.y));
-                    const float2 h23 = ptx::silu_fast2(make_float2(__uint_as_float(v[k0 + 2]), __uint_as_float(v[k0 + 3])),
+                    const float2 h23 = ptx::silu_bias2(make_float2(__uint_as_float(v[k0 + 2]), __uint_as_float(v[k0 + 3])),
                                                        make_float2(b.z, b.w));
                     ca = fmaf(xa.x, h01.x, ca), cp = fmaf(xq.x, h01.x, cp);
                     ca = fmaf(xa.y, h01.y, ca), cp = fmaf(xq.y, h01.y, cp);
                     ca = fmaf(xa.z, h23.x, ca), cp = fmaf(xq.z, h23.x, cp);
                     ca = fmaf(xa.w, h23.y, ca), cp = fmaf(xq.w, h23.y, cp);
                 }
-                const int idx = wide_contrib(pl, x) + y * G + g;
+                const int idx = wide_contrib(pl, x) + w.y * pl.G + w.g;
                 contrib[idx] = ca;
-                contrib[idx + L * G] = cp;
+                contrib[idx + L * pl.G] = cp;
             }
         }
     }
@@ -1213,44 +1432,63 @@ __device__ bool wide_epilogue(const TcPlan &pl, const TcShared &sh, uint32_t &ph
 }
 
 // Sums of the head contributions per configuration, in head_slot's order
-// (lane k takes sites k, k + 32, ..., then the xor-shuffle tree); one warp per
-// configuration and output.
-__device__ void wide_head(const TcPlan &pl, const TcShared &sh) {
+// (lane k takes the original sites k, k + 32, ..., then the xor-shuffle tree);
+// one warp per configuration and output.
+__device__ void wide_head(const TcPlan &pl, const TcShared &sh, const WideCfg *cfgs) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = pl.G, L = pl.L;
     const float *contrib = reinterpret_cast<const float *>(sh.base + pl.o_act);
+    const int y0 = lane / L, x0 = lane - y0 * L, dy = 32 / L, dx = 32 - dy * L, colw = pl.Lp * G * 4 + 1;
     for (int t = warp; t < 2 * G; t += (int)(blockDim.x >> 5)) {
-        const int g = t >> 1, o = t & 1;
+        const int g = t >> 1;
+        const float *src = contrib + (t & 1) * L * G + g;
+        int c = x0 - cfgs[g].roll, y = y0;   // canonical column, row of the lane's site
+        if (c < 0) c += L;
+        int x = x0;
         float sum = 0.f;
         for (int site = lane; site < pl.N; site += 32) {
-            const int y = site / L, x = site - y * L;
-            sum += contrib[wide_contrib(pl, x) + o * L * G + y * G + g];
+            sum += src[c * colw + y * G];
+            x += dx, y += dy, c += dx;
+            if (c >= L) c -= L;
+            if (x >= L) { x -= L; ++y; }
         }
 #pragma unroll
         for (int k = 16; k > 0; k >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, k);
-        if (lane == 0) sh.res[o * G + g] = (double)sum;
+        if (lane == 0) sh.res[(t & 1) * G + g] = (double)sum;
     }
     __syncthreads();
 }
 
-// Evaluate the group's G configurations (sh.spins) in the wide row form;
-// results in sh.res. False if a wait gave up (the block must stop).
+// Evaluate the group's G configurations (cfgs, of the sample sigma) in the
+// wide row form; results in sh.res. False if a wait gave up (the block must
+// stop).
 template <int C>
-__device__ bool wide_forward(const TcPlan &pl, const TcShared &sh, const unsigned char *packed, TcState &st, int *err) {
-    build_rows(pl, sh);
-    const int warp = threadIdx.x >> 5, nl = pl.n_layers;
+__device__ bool wide_forward(const TcPlan &pl, const TcShared &sh, const unsigned char *packed, TcState &st, int *err,
+                             const int8_t *sigma, const WideCfg *cfgs, int cls, const unsigned char *cache,
+                             unsigned char *cache_w) {
+    {
+        int lo, hi;
+        wide_cols(pl, cls, 0, lo, hi);
+        wide_build(pl, sh, sigma, cfgs, lo, hi);
+    }
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), nl = pl.n_layers;
     uint32_t ph = st.tphase;
     bool ok = true;
-    if (warp >= pl.epi) {
+    if (warp >= pl.epi + kIssuers) {
+        for (int l = 0; ok && l < nl; ++l)
+            ok = wide_fill_layer<C>(pl, sh, ph, l, cls, cfgs, cache, warp - pl.epi - kIssuers);
+    } else if (warp >= pl.epi) {
         const int iw = warp - pl.epi;
         for (int l = 0; ok && l < nl; ++l) {
-            if (l > 0) {   // stage 1 + iw of the layer before: this half's input is written, its accumulators drained
-                ok = __all_sync(0xffffffffu, wait_or_abort(&sh.bar_tile[2 + iw], (ph >> (2 + iw)) & 1u, sh.abort_flag));
+            if (l > 0) {   // stage 1 (A) or 2 (B) of the layer before: this half's input is written, its accumulators drained
+                ok = __all_sync(0xffffffffu,
+                                wide_wait(&sh.bar_tile[2 + iw], (ph >> (2 + iw)) & 1u, sh.abort_flag));
                 ph ^= 4u << iw;
             }
-            ok = ok && wide_issue<C>(pl, sh, packed, st, l, iw);
+            ok = ok && wide_issue<C>(pl, sh, packed, st, l, iw, cls);
         }
     } else {
-        for (int l = 0; ok && l < nl; ++l) ok = wide_epilogue<C>(pl, sh, ph, l, err);
+        const WideRow w = wide_row(pl, sh, threadIdx.x & 127);
+        for (int l = 0; ok && l < nl; ++l) ok = wide_epilogue<C>(pl, sh, w, ph, l, err, cls, cache_w);
     }
     if (!ok) raise_abort(sh, err);
     // every thread leaves with the same barrier phases: A and B complete nl times, the stages nl - 1 times
@@ -1260,8 +1498,135 @@ __device__ bool wide_forward(const TcPlan &pl, const TcShared &sh, const unsigne
     __syncthreads();
     ptx::tc_fence_after();
     if (*(volatile int *)sh.abort_flag) return false;
-    wide_head(pl, sh);
+    wide_head(pl, sh, cfgs);
     st.wseq += (uint32_t)nl;
+    return true;
+}
+
+// Shared memory of wide_sample after the plan's arrays: the sample, its
+// connected list, the log psi of every entry as the float32 sums the head
+// makes, the evaluation order and the group's configurations.
+struct WideExtra {
+    int8_t *sigma;
+    int16_t *ci, *cj, *ord;
+    double *ch, *fsum;
+    int *cum;
+    EnumScratch *scr;
+    float *lp;       // [chunk + 1][2]
+    WideCfg *cfgs;   // [16]
+};
+
+__host__ __device__ inline WideExtra wide_extra(unsigned char *ex, int N, int chunk, uint32_t *bytes) {
+    WideExtra e;
+    uint32_t o = 0;
+    e.ch = reinterpret_cast<double *>(ex + o); o += 8 * chunk;
+    e.fsum = reinterpret_cast<double *>(ex + o); o += 8 * 258;
+    e.scr = reinterpret_cast<EnumScratch *>(ex + o); o = al16(o + (uint32_t)sizeof(EnumScratch));
+    e.lp = reinterpret_cast<float *>(ex + o); o += 8 * (chunk + 1);
+    e.cfgs = reinterpret_cast<WideCfg *>(ex + o); o += 16 * (uint32_t)sizeof(WideCfg);
+    e.cum = reinterpret_cast<int *>(ex + o); o += 4 * (N + 1);
+    e.ci = reinterpret_cast<int16_t *>(ex + o); o += 2 * chunk;
+    e.cj = reinterpret_cast<int16_t *>(ex + o); o += 2 * chunk;
+    e.ord = reinterpret_cast<int16_t *>(ex + o); o += 2 * chunk;
+    e.sigma = reinterpret_cast<int8_t *>(ex + o); o += N;
+    *bytes = al16(o);
+    return e;
+}
+
+// Local energy of one configuration through the wide row form: as eloc_sample
+// (the same terms in the same fixed order), with the group's configurations
+// described by their exchange and roll instead of copied.
+template <int C>
+__device__ bool wide_sample(const TcPlan &pl, const Problem &p, const TcShared &sh, TcState &st,
+                            const unsigned char *packed, const int8_t *cfg, const double *logpsi_s, double *out_s,
+                            int *err, unsigned char *cache) {
+    const int G = pl.G, N = pl.N, L = pl.L, chunk = bond_chunk(p);
+    uint32_t bytes;
+    const WideExtra e = wide_extra(sh.base + pl.o_extra, N, chunk, &bytes);
+    const int recompute = logpsi_s == nullptr;
+    // cones need the sample's own activations, so only where it is evaluated here
+    const bool cone = cache != nullptr && recompute;
+    for (int r = threadIdx.x; r < N; r += blockDim.x) e.sigma[r] = cfg[r];
+    __syncthreads();
+    if (p.model == NQS_MODEL_TJ) snake_prefix(p, e.sigma, e.cum, *e.scr);
+    double ref_a = 0.0, ref_phi = 0.0, hd_tot = 0.0, sr_tot = 0.0, si_tot = 0.0;   // identical in every thread
+    if (!recompute) { ref_a = logpsi_s[0]; ref_phi = logpsi_s[1]; }
+    for (int b0 = 0; b0 < p.n_bonds; b0 += chunk) {
+        double hd;
+        const int nconn = enumerate_range(p, e.sigma, b0, min(p.n_bonds, b0 + chunk), e.ci, e.cj, e.ch, &hd, e.cum,
+                                          *e.scr);
+        hd_tot += hd;
+        const int lead = (recompute && b0 == 0) ? 1 : 0;   // sigma itself evaluated first
+        const int n_entries = nconn + lead;
+        // evaluation order: the first group (sigma and G - 1 entries) in list order; with cones the other entries
+        // by class (pair in one column, then in two), stable, so that a group shares its band
+        const int first = cone ? min(nconn, G - lead) : nconn;
+        for (int k = threadIdx.x; k < first; k += blockDim.x) e.ord[k] = (int16_t)k;
+        int base = first;
+        for (int cls = 0; cls < 2 && first < nconn; ++cls)
+            for (int k0 = first; k0 < nconn; k0 += blockDim.x) {
+                const int k = k0 + threadIdx.x;
+                const int f = k < nconn && (int)(e.ci[k] % L != e.cj[k] % L) == cls;
+                int tot;
+                const int off = block_exclusive_scan(f, e.scr->iscr, &tot);
+                if (f) e.ord[base + off] = (int16_t)k;
+                base += tot;
+            }
+        __syncthreads();
+        for (int e0 = 0; e0 < n_entries; e0 += G) {
+            const int cnt = min(G, n_entries - e0);
+            // the group's class is its last entry's (class 1's band covers class 0); dense if it holds the sample
+            int cls = -1;
+            if (cone && e0 >= lead + first) {
+                const int k = e.ord[e0 + cnt - 1 - lead];
+                cls = e.ci[k] % L != e.cj[k] % L;
+            }
+            if (threadIdx.x < G) {
+                const int c = threadIdx.x, q = e0 + c - lead;   // list position (-1: sigma)
+                WideCfg v{-1, -1, 0, 0};
+                if (c < cnt && q >= 0) {
+                    const int k = e.ord[q];
+                    if (NQS_INDEX_OK(k >= 0 && k < nconn && e.ci[k] >= 0 && e.ci[k] < N && e.cj[k] >= 0 && e.cj[k] < N,
+                                     err)) {
+                        v.i = e.ci[k];
+                        v.j = e.cj[k];
+                        if (cls >= 0) {   // the bond's first site is the left one: to column H - 1
+                            const int r = v.i % L - (L / 2 - 1);
+                            v.roll = (int16_t)(r < 0 ? r + L : r);
+                        }
+                    }
+                }
+                e.cfgs[c] = v;
+            }
+            __syncthreads();
+            if (!wide_forward<C>(pl, sh, packed, st, err, e.sigma, e.cfgs, cls, cache,
+                                 cone && lead && e0 == 0 ? cache : nullptr))
+                return false;
+            if (threadIdx.x < cnt) {
+                const int q = e0 + (int)threadIdx.x - lead, idx = q < 0 ? 0 : e.ord[q] + lead;
+                e.lp[2 * idx] = (float)sh.res[threadIdx.x];
+                e.lp[2 * idx + 1] = (float)sh.res[G + threadIdx.x];
+            }
+        }
+        __syncthreads();
+        if (lead) { ref_a = (double)e.lp[0]; ref_phi = (double)e.lp[1]; }
+        // off-diagonal terms in an order independent of the block size
+        const double2 tsum = fixed_order_sum2(nconn, [&](int k) {
+            const double m = e.ch[k] * exp((double)e.lp[2 * (k + lead)] - ref_a);
+            double sn, cs;
+            sincos((double)e.lp[2 * (k + lead) + 1] - ref_phi, &sn, &cs);
+            return make_double2(m * cs, m * sn);
+        }, e.fsum);
+        sr_tot += tsum.x;
+        si_tot += tsum.y;
+    }
+    if (threadIdx.x == 0) {
+        const double er = hd_tot + sr_tot, ei = si_tot;
+        out_s[0] = er;
+        out_s[1] = ei;
+        if (!isfinite(er) || !isfinite(ei)) atomicOr(err, ERRBIT_NONFINITE);
+    }
+    __syncthreads();
     return true;
 }
 
@@ -1278,7 +1643,7 @@ __device__ void tc_init(TcShared &sh, unsigned char *smem, uint32_t tmem_cols, T
         ptx::mbar_init(&sh.bar_w[0], 1);
         ptx::mbar_init(&sh.bar_w[1], 1);
         for (int t = 0; t < kMaxSlots * kMaxTiles; ++t)
-            ptx::mbar_init(&sh.bar_tile[t], (t == 2 || t == 3) ? stage_arrivals : 1u);
+            ptx::mbar_init(&sh.bar_tile[t], t == 2 || t == 3 ? stage_arrivals : 1u);
         *sh.abort_flag = 0;
         ptx::fence_mbar_init();
     }
@@ -1339,8 +1704,8 @@ __device__ void tc_bind(const TcPlan &pl, TcShared &sh, const unsigned char *pac
     st.wissued += 1;
 }
 
-// Bind the block to a row-form plan (either form): parameters, MMA lists,
-// zeroed activations and zero block, first weight load.
+// Bind the block to a row-form plan (either form): parameters, the row
+// form's MMA lists, zeroed activations and zero block, first weight load.
 __device__ void row_bind(const TcPlan &pl, TcShared &sh, const unsigned char *packed, TcState &st) {
     unsigned char *smem = sh.base;
     sh.spins = reinterpret_cast<int8_t *>(smem + pl.o_spins);
@@ -1349,18 +1714,28 @@ __device__ void row_bind(const TcPlan &pl, TcShared &sh, const unsigned char *pa
     sh.f32 = reinterpret_cast<float *>(smem + pl.o_f32);
     sh.res = reinterpret_cast<double *>(smem + pl.o_res);
     const float *src = reinterpret_cast<const float *>(packed);
-    for (uint32_t i = threadIdx.x; i < pl.f32_count; i += blockDim.x) sh.f32[i] = src[i];
+    // the wide form's epilogue reads halved biases
+    const uint32_t halved = pl.rows == 2 ? (uint32_t)(pl.n_layers * pl.C) : 0u;
+    for (uint32_t i = threadIdx.x; i < pl.f32_count; i += blockDim.x) sh.f32[i] = i < halved ? 0.5f * src[i] : src[i];
+    if (pl.rows == 2)
+        for (int m = threadIdx.x; m < 128; m += blockDim.x) {
+            const bool valid = m < pl.G * pl.L;
+            const int y = valid ? m / pl.G : 0, g = valid ? m - y * pl.G : 0;
+            const int yimg = y == 0 ? pl.L + 1 : (y == pl.L - 1 ? 0 : -1);
+            reinterpret_cast<int4 *>(smem + pl.o_lane)[m] =
+                make_int4(y | (g << 8) | ((int)valid << 16), ((y + 1) * pl.G + g) * 16,
+                          yimg < 0 ? 0 : (yimg - (y + 1)) * pl.G * 16, 0);
+        }
     // zero the activations (rows no output writes are read only by discarded
     // accumulator rows, but stay finite) and the zero block
     for (uint32_t i = threadIdx.x; i < pl.act_bytes / 4; i += blockDim.x)
         reinterpret_cast<uint32_t *>(smem + pl.o_act)[i] = 0u;
     const uint32_t zero = pl.rows == 2 ? kZeroWide : kZeroRows;
     for (uint32_t i = threadIdx.x; i < zero / 4; i += blockDim.x) reinterpret_cast<uint32_t *>(smem + pl.o_zero)[i] = 0u;
-    {
+    if (pl.rows == 1) {
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, iw = warp - pl.epi;
         if (lane == 0 && iw >= 0 && iw < kIssuers) {
-            if (pl.rows == 2) wide_build_mtab<32>(pl, sh, iw);
-            else if (pl.C == 16) row_build_mtab<16>(pl, sh, iw);
+            if (pl.C == 16) row_build_mtab<16>(pl, sh, iw);
             else row_build_mtab<32>(pl, sh, iw);
         }
     }
@@ -1448,9 +1823,8 @@ __global__ void __launch_bounds__(kTcThreads, kMinBlocks<C>) logpsi_tc_kernel(Tc
 // configurations, evaluate sigma and all of them in groups, then
 // E_loc = H_diag + sum_k H_k exp((a'_k - a) + i (phi'_k - phi)) in float64,
 // every term of the sample at once, fixed-order block reduction.
-// FORM: the forward the configurations go through (0 tap form, with cones if
-// there is a cache; 1 row form, 2 wide row form, both dense).
-template <int C, int FORM = 0, bool F8 = false>
+// ROWS: the configurations go through the row form (no cones).
+template <int C, bool ROWS = false, bool F8 = false>
 __device__ bool eloc_sample(const TcPlan &pl, const Problem &p, const TcShared &sh, TcState &st,
                             const unsigned char *packed, const int8_t *cfg, const double *logpsi_s, double *out_s,
                             int *err, unsigned char *cache) {
@@ -1464,15 +1838,14 @@ __device__ bool eloc_sample(const TcPlan &pl, const Problem &p, const TcShared &
     EnumScratch *scr = reinterpret_cast<EnumScratch *>(ex + al16(N) + al16(4 * chunk) + al16(8 * chunk) +
                                                        al16(4 * (N + 1)));
     double *ref = reinterpret_cast<double *>(scr + 1);   // a0, phi0
-    float *lp = reinterpret_cast<float *>(ref + 4);       // [chunk + 1][2]: (a, phi) of every list entry (the head's
-                                                          // float32 sums, so the float keeps every bit)
-    double *fsum = ref + 4 + (chunk + 1);                 // [258] fixed-order sum scratch
+    double *lp = ref + 4;                                 // [chunk + 1][2]: (a, phi) of every list entry
+    double *fsum = lp + 2 * (chunk + 1);                  // [258] fixed-order sum scratch
     int16_t *ord = reinterpret_cast<int16_t *>(fsum + 258);   // [chunk] evaluation order of the entries
     int *roll = reinterpret_cast<int *>(ord + ((chunk + 1) & ~1));   // [32] per configuration of a group
     const int recompute = logpsi_s == nullptr;
     // the cone of every connected configuration is evaluated alone when the
     // sample itself is evaluated here (its activations fill the cache)
-    const bool cone = FORM == 0 && cache != nullptr && recompute && pl.slots == 1;
+    const bool cone = !ROWS && cache != nullptr && recompute && pl.slots == 1;
     for (int r = threadIdx.x; r < N; r += blockDim.x) sigma[r] = cfg[r];
     __syncthreads();
     if (p.model == NQS_MODEL_TJ) snake_prefix(p, sigma, cum, *scr);
@@ -1553,9 +1926,7 @@ __device__ bool eloc_sample(const TcPlan &pl, const Problem &p, const TcShared &
                 }
             }
             __syncthreads();
-            if constexpr (FORM == 2) {
-                if (!wide_forward<C>(pl, sh, packed, st, err)) return false;
-            } else if constexpr (FORM == 1) {
+            if (ROWS) {
                 if (!row_forward<C, F8>(pl, sh, packed, st, err)) return false;
             } else if (!tc_forward<C>(pl, sh, packed, st, err, band, cache, (cone && lead && e0 == 0) ? cache : nullptr)) {
                 return false;
@@ -1564,8 +1935,8 @@ __device__ bool eloc_sample(const TcPlan &pl, const Problem &p, const TcShared &
                 const int c = threadIdx.x, sl = c / G, g = c - sl * G;
                 const int q = e0 + c - lead;
                 const int idx = q < 0 ? 0 : ord[q] + lead;
-                lp[2 * idx] = (float)sh.res[sl * 2 * G + g];
-                lp[2 * idx + 1] = (float)sh.res[sl * 2 * G + G + g];
+                lp[2 * idx] = sh.res[sl * 2 * G + g];
+                lp[2 * idx + 1] = sh.res[sl * 2 * G + G + g];
             }
             __syncthreads();
         }
@@ -1574,9 +1945,9 @@ __device__ bool eloc_sample(const TcPlan &pl, const Problem &p, const TcShared &
         __syncthreads();
         // off-diagonal terms in an order independent of the block size
         const double2 tsum = fixed_order_sum2(nconn, [&](int k) {
-            const double m = ch[k] * exp((double)lp[2 * (k + lead)] - ref[0]);
+            const double m = ch[k] * exp(lp[2 * (k + lead)] - ref[0]);
             double sn, cs;
-            sincos((double)lp[2 * (k + lead) + 1] - ref[1], &sn, &cs);
+            sincos(lp[2 * (k + lead) + 1] - ref[1], &sn, &cs);
             return make_double2(m * cs, m * sn);
         }, fsum);
         sr_tot += tsum.x;
@@ -1620,25 +1991,26 @@ __global__ void __launch_bounds__(kTcThreads, 2)
     tc_init(sh, smem, pl.tmem_cols, st);
     row_bind(pl, sh, packed, st);
     for (int64_t s = blockIdx.x; s < n; s += gridDim.x)
-        if (!eloc_sample<C, 1, F8>(pl, p, sh, st, packed, configs + s * p.N, logpsi ? logpsi + 2 * s : nullptr,
+        if (!eloc_sample<C, true, F8>(pl, p, sh, st, packed, configs + s * p.N, logpsi ? logpsi + 2 * s : nullptr,
                                       out + 2 * s, err, nullptr))
             break;
     tc_teardown(pl, sh, st);
 }
 
-// Local energies through the wide row form (32 channels, one block per SM).
+// Local energies through the wide row form (16 channels: two blocks per SM).
 template <int C>
-__global__ void __launch_bounds__(kWideThreads, 1)
+__global__ void __launch_bounds__(kWideThreads<C>, kWideBlocks<C>)
     eloc_wide_kernel(TcPlan pl, Problem p, const unsigned char *packed, const int8_t *configs, const double *logpsi,
-                     int64_t n, double *out, int *err) {
+                     int64_t n, double *out, int *err, unsigned char *cache) {
     extern __shared__ __align__(128) unsigned char smem[];
     TcShared sh;
     TcState st;
-    tc_init(sh, smem, pl.tmem_cols, st, (uint32_t)pl.epi);
+    tc_init(sh, smem, pl.tmem_cols, st, (blockDim.x >> 5) - kIssuers);   // epilogue and fill warps
     row_bind(pl, sh, packed, st);
+    unsigned char *my_cache = cache ? cache + (size_t)blockIdx.x * wide_cache_bytes(pl) : nullptr;
     for (int64_t s = blockIdx.x; s < n; s += gridDim.x)
-        if (!eloc_sample<C, 2>(pl, p, sh, st, packed, configs + s * p.N, logpsi ? logpsi + 2 * s : nullptr, out + 2 * s,
-                               err, nullptr))
+        if (!wide_sample<C>(pl, p, sh, st, packed, configs + s * p.N, logpsi ? logpsi + 2 * s : nullptr, out + 2 * s,
+                            err, my_cache))
             break;
     tc_teardown(pl, sh, st);
 }
@@ -2024,14 +2396,16 @@ bool make_row_plan(const Problem &p, size_t max_smem, int extra_bytes, TcPlan *o
     return true;
 }
 
-// Wide row-form plan (32 channels): G = min(16, 128 / L) configurations per
-// block, one block per SM, up to all 512 accumulator columns.
-bool make_wide_plan(const Problem &p, size_t max_smem, int extra_bytes, TcPlan *out, std::string *why, int G = 0) {
-    if (p.C != 32 || p.L * p.C > 512) { *why = "wide row form: 32 channels, L * C <= 512"; return false; }
+// Wide row-form plan: G = min(16, 128 / L) configurations per block; 16
+// channels: two blocks per SM, 32 channels: one block and up to all 512
+// accumulator columns.
+bool make_wide_plan(const Problem &p, size_t max_smem, TcPlan *out, std::string *why, int G = 0) {
+    const int ctas = p.C == 16 ? 2 : 1;
+    if (p.L * p.C * ctas > 512) { *why = "wide row form: accumulators exceed tensor memory"; return false; }
     TcPlan pl{};
     pl.rows = 2;
-    pl.ctas = 1;
-    pl.epi = kWideEpi;
+    pl.ctas = ctas;
+    pl.epi = ctas == 2 ? kMaxEpiWarps : kWideEpi;
     pl.L = p.L;
     pl.Lp = p.L + 2;
     pl.N = p.N;
@@ -2047,10 +2421,11 @@ bool make_wide_plan(const Problem &p, size_t max_smem, int extra_bytes, TcPlan *
     // activations x Lp G + yp G + g; the last A operand starts 2 G rows into column L - 1 and spans 128 rows; the
     // im2col of layer 0 takes L x 128
     pl.rows_total = std::max(p.L * pl.Lp * pl.G + 128 - p.L * pl.G, p.L * 128);
-    pl.rows_total = (pl.rows_total + 7) & ~7;
+    // the planes of one row fall on different banks (8 / KC 16-byte groups apart), for the copies of wide_fill
+    pl.rows_total = (pl.rows_total + 7) / 8 * 8 + 8 / pl.KC;
     pl.rbuf = pl.rows_total;
     pl.plane = (uint32_t)pl.rows_total * 16u;
-    pl.act_bytes = pl.plane * (uint32_t)pl.KC;
+    pl.act_bytes = pl.plane * (uint32_t)std::max(pl.KC, pl.K0 / 8);
     pl.slot_cols = (uint32_t)(p.L * p.C);
     uint32_t cols = 32;
     while (cols < pl.slot_cols) cols <<= 1;
@@ -2062,14 +2437,19 @@ bool make_wide_plan(const Problem &p, size_t max_smem, int extra_bytes, TcPlan *
     pl.o_w0 = o; o = al16(o + pl.wbytes);
     pl.o_w1 = o; o = al16(o + pl.wbytes);
     pl.o_f32 = o; o = al16(o + pl.f32_count * 4);
-    pl.o_mtab = o; o = al16(o + kMtabBytes);
-    pl.o_spins = o; o = al16(o + pl.G * p.N);
+    pl.o_lane = o; o = al16(o + 16 * 128);
     pl.o_res = o; o = al16(o + 16 * pl.G);
-    pl.o_extra = o; o = al16(o + extra_bytes);
+    uint32_t extra;
+    wide_extra(nullptr, p.N, bond_chunk(p), &extra);
+    pl.o_extra = o; o = al16(o + extra);
     const uint32_t sm_bytes = 233472u;   // 228 KB per SM, 1 KB reserved per block
-    while (cols * (sm_bytes / (o + 1024u)) > 512u || 2u * (o + 1024u) <= sm_bytes) o += 1024u;   // one block per SM
+    // no more co-resident blocks than planned (tensor memory would not serve them)
+    while (sm_bytes / (o + 1024u) > (uint32_t)ctas) o += 1024u;
     pl.total = o;
-    if (pl.total > max_smem) { *why = "wide row form: shared memory plan exceeds the per-block limit"; return false; }
+    if ((uint32_t)ctas * (pl.total + 1024u) > sm_bytes || pl.total > max_smem) {
+        *why = "wide row form: shared memory plan exceeds the limit";
+        return false;
+    }
     *out = pl;
     return true;
 }
@@ -2077,7 +2457,7 @@ bool make_wide_plan(const Problem &p, size_t max_smem, int extra_bytes, TcPlan *
 // Whether the local-energy launch uses the row form (NQS_TC_ROWS=0 turns it
 // off, NQS_TC_ROWS=G forces G configurations per group: tuning and A/B
 // comparisons).
-bool use_row_form(const Problem &p, size_t max_smem, TcPlan *out) {
+bool use_row_form(const Problem &p, size_t max_smem, bool f8, TcPlan *out) {
     const char *e = getenv("NQS_TC_ROWS");
     int G = 0;
     if (e) {
@@ -2085,8 +2465,15 @@ bool use_row_form(const Problem &p, size_t max_smem, TcPlan *out) {
         if (G == 0) return false;
     }
     std::string why;
-    return make_row_plan(p, max_smem, eloc_extra(p), out, &why, G) ||
-           make_wide_plan(p, max_smem, eloc_extra(p), out, &why, G);
+    const bool rows = make_row_plan(p, max_smem, eloc_extra(p), out, &why, G);
+    if (f8) return rows;
+    // The wide form where it is the faster one (GB300, ms, wide / the other form; 2,432 samples at 16 channels, 1,216
+    // at 32). 16 channels, against the row form: from three layers on 8 x 8 and larger and four on smaller lattices
+    // (10x10: 1.61 / 1.59 with two layers, 2.49 / 2.68 with four, 4.23 / 4.78 with eight; 6x6: 0.46 / 0.43, 0.68 /
+    // 0.68, 1.12 / 1.17). 32 channels, against the tap form: from 6 x 6 (5x5, four layers 0.51 / 0.49; 6x6 0.72 /
+    // 0.79; 10x10 2.64 / 4.15; 16x16, eight layers, cones in both: 20.1 / 37.6).
+    if (p.C == 16 ? !rows || p.n_layers < (p.L >= 8 ? 3 : 4) : p.L < 6) return rows;
+    return make_wide_plan(p, max_smem, out, &why, G) || rows;
 }
 
 bool make_plan(const Problem &p, int G, int slots, int ctas, size_t max_smem, int extra_bytes, TcPlan *out,
@@ -2144,7 +2531,7 @@ bool make_plan(const Problem &p, int G, int slots, int ctas, size_t max_smem, in
 int eloc_extra(const Problem &p) {
     const int chunk = bond_chunk(p);
     return (int)(al16(p.N) + al16(4 * chunk) + al16(8 * chunk) + al16(4 * (p.N + 1)) + sizeof(EnumScratch) +
-                 4 * sizeof(double) + 8 * (chunk + 1) + 8 * 258 + 2 * ((chunk + 1) & ~1) + 4 * 32);
+                 4 * sizeof(double) + 16 * (chunk + 1) + 8 * 258 + 2 * ((chunk + 1) & ~1) + 4 * 32);
 }
 
 int sample_extra(const Problem &p, int G, int slots) {
@@ -2282,11 +2669,16 @@ int launch_logpsi_tc(const Problem &p, const double *, const void *packed, const
 size_t tc_eloc_cache_bytes(const Problem &p, size_t max_smem, int num_sms, int64_t n) {
     std::string why;
     TcPlan pl;
-    if (n <= 0 || !tc_supported(p, &why) || use_row_form(p, max_smem, &pl) ||
-        !best_plan(p, max_smem, true, 16, 2, &pl, &why))
-        return 0;
+    if (n <= 0 || !tc_supported(p, &why)) return 0;
     const char *d = getenv("NQS_TC_DENSE"), *f = getenv("NQS_TC_CONES");
     const bool force = f && f[0] == '1';
+    if (use_row_form(p, max_smem, false, &pl)) {
+        // wide form, 32 channels: a narrow band still pays a layer's three stages, so the cones pay from 15 x 15
+        // (measured with eight layers, cones / dense: 16x16 20.1 / 22.4 ms, 15x15 17.2 / 18.5, 14x14 15.4 / 14.5)
+        if (pl.rows != 2 || pl.ctas != 1 || p.n_layers < 2 || (d && d[0] == '1') || (p.L < 15 && !force)) return 0;
+        return (size_t)std::min<int64_t>(n, (int64_t)num_sms * pl.ctas) * wide_cache_bytes(pl);
+    }
+    if (!best_plan(p, max_smem, true, 16, 2, &pl, &why)) return 0;
     if (pl.slots != 1 || p.n_layers < 2 || (d && d[0] == '1') || (pl.ctas != 1 && !force)) return 0;
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)num_sms * pl.ctas));
     return (size_t)grid * sigma_cache_bytes(pl);
@@ -2305,7 +2697,7 @@ int launch_eloc_tc(const Problem &p, const double *, const void *packed, const i
     if (f8) {
         // e4m3 operands: the row form with 16 channels; the sample's log psi is always recomputed, so that
         // every ratio of the local energy is taken in the same arithmetic
-        if (p.C != 16 || !use_row_form(p, env.max_smem, &pl)) {
+        if (p.C != 16 || !use_row_form(p, env.max_smem, true, &pl)) {
             *env.msg = "e4m3 local energies need the row form with 16 channels";
             return NQS_ERR_UNSUPPORTED;
         }
@@ -2319,13 +2711,18 @@ int launch_eloc_tc(const Problem &p, const double *, const void *packed, const i
                                                                     nullptr, n, out, env.err);
         return check(env, "eloc_rows_kernel (e4m3)");
     }
-    if (use_row_form(p, env.max_smem, &pl)) {
+    if (use_row_form(p, env.max_smem, false, &pl)) {
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)env.num_sms * pl.ctas));
         if (pl.rows == 2) {
-            auto k = eloc_wide_kernel<32>;
-            if (int rc = prep(k, pl, env)) return rc;
-            k<<<grid, 32 * (pl.epi + kIssuers), pl.total, env.stream>>>(pl, p, (const unsigned char *)packed, configs,
-                                                                        logpsi, n, out, env.err);
+            const size_t need = tc_eloc_cache_bytes(p, env.max_smem, env.num_sms, n);
+            unsigned char *c = (need > 0 && cache && cache_bytes >= need) ? (unsigned char *)cache : nullptr;
+            const int threads = 32 * (pl.epi + kIssuers + (c ? kWideFill : 0));
+            NQS_TC_DISPATCH(p.C, {
+                auto k = eloc_wide_kernel<CC>;
+                if (int rc = prep(k, pl, env)) return rc;
+                k<<<grid, threads, pl.total, env.stream>>>(pl, p, (const unsigned char *)packed, configs, logpsi,
+                                                                    n, out, env.err, c);
+            });
             return check(env, "eloc_wide_kernel");
         }
         NQS_TC_DISPATCH(p.C, {
@@ -2486,7 +2883,7 @@ int tc_describe_plan(const Problem &p, int kind, int64_t n, size_t max_smem, int
     bool ok = tc_supported(p, why);
     if (ok) {
         if (kind == 2) ok = sample_plan(p, max_smem, &pl, why);
-        else if (kind == 1 && use_row_form(p, max_smem, &pl)) ok = true;
+        else if (kind == 1 && use_row_form(p, max_smem, false, &pl)) ok = true;
         else ok = best_plan(p, max_smem, kind == 1, 16, 2, &pl, why);
     }
     if (!ok) return NQS_ERR_UNSUPPORTED;

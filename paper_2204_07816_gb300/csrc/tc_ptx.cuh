@@ -52,6 +52,27 @@ __device__ __forceinline__ bool mbar_try_wait_sleep(uint64_t *bar, uint32_t pari
     return ok != 0;
 }
 
+// Up to `polls` tests in a tight loop (three instructions a poll: warps that
+// wait beside working ones should take few issue slots).
+__device__ __forceinline__ bool mbar_poll(uint64_t *bar, uint32_t parity, uint32_t polls) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\t"
+        "mov.u32 n, %3;\n"
+        "POLL_%=:\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra DONE_%=;\n\t"
+        "sub.u32 n, n, 1;\n\t"
+        "setp.ne.u32 q, n, 0;\n\t"
+        "@q bra POLL_%=;\n"
+        "DONE_%=:\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(polls)
+        : "memory");
+    return ok != 0;
+}
+
 // Nanosecond timer (global, monotonic).
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
@@ -179,6 +200,17 @@ __device__ __forceinline__ void mma_e4m3_elect(uint32_t d_tmem, uint64_t adesc, 
         : "memory");
 }
 
+// One lane of a converged warp (the same lane in every call).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, e;\n\t}\n"
+        : "=r"(ok));
+    return ok != 0;
+}
+
 // Commit of the MMAs issued through mma_bf16_elect (elect.sync's choice over
 // a full warp is deterministic, so the committing lane is the issuing one).
 // Every lane must execute it.
@@ -264,6 +296,31 @@ __device__ __forceinline__ float2 silu_fast2(float2 v, float2 b) {
     return silu_half2(__fmul2_rn(make_float2(0.5f, 0.5f), __fadd2_rn(v, b)));
 }
 
+// SiLU(v + b) of 16 accumulators given the halved biases, packed to bf16
+// pairs: the 16 tanh instructions are issued back to back (volatile keeps
+// them together), so their latency is paid once and not per pair. Bitwise
+// silu_bias2 and pack_bf16.
+__device__ __forceinline__ float tanh_approx_ordered(float x) {
+    float y;
+    asm volatile("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi);
+__device__ __forceinline__ void silu_bias16(const uint32_t (&r)[16], const float (&hb)[16], uint32_t (&o)[8]) {
+    float2 hz[8], t[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+        hz[c] = __ffma2_rn(make_float2(0.5f, 0.5f), make_float2(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])),
+                           make_float2(hb[2 * c], hb[2 * c + 1]));
+#pragma unroll
+    for (int c = 0; c < 8; ++c) t[c] = make_float2(tanh_approx_ordered(hz[c].x), tanh_approx_ordered(hz[c].y));
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float2 v = __ffma2_rn(hz[c], t[c], hz[c]);
+        o[c] = pack_bf16(v.x, v.y);
+    }
+}
+
 // Two floats to e4m3 (round to nearest even, saturating to +-448), lo in the
 // low byte of the 16-bit result.
 __device__ __forceinline__ uint32_t pack_e4m3(float lo, float hi) {
@@ -283,6 +340,11 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 __device__ __forceinline__ void cp_async16(uint32_t dst_smem, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst_smem), "l"(src) : "memory");
 }
+
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Wait until at most N of this thread's committed groups are pending.
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 

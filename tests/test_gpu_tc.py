@@ -163,6 +163,41 @@ def test_local_energy_row_form_equals_tap_form(case, give_logpsi, monkeypatch):
     assert abs(got[:, 0].mean() - want.real.mean()) / L ** 2 <= 1e-4
 
 
+WIDE_CASES = [
+    ('j1j2_16x16', {'n_layers': 4}),
+    ('j1j2_16x16', {'L': 15, 'n_up': 113, 'n_down': 112, 'n_layers': 7}),
+    ('j1j2_16x16', {'L': 13, 'n_up': 85, 'n_down': 84, 'n_layers': 2}),
+    ('j1j2_16x16', {'L': 9, 'n_up': 41, 'n_down': 40, 'n_layers': 3}),
+    ('j1j2_16x16', {'L': 6, 'n_up': 18, 'n_down': 18, 'n_layers': 1}),
+    ('tj_12x12', {}),
+    ('tj_12x12', {'L': 16, 'n_up': 112, 'n_down': 112, 'n_layers': 8}),
+    ('tj_12x12', {'L': 7, 'n_up': 22, 'n_down': 21, 'n_layers': 5}),
+]
+
+
+@pytest.mark.parametrize('case', WIDE_CASES, ids=_ids)
+def test_local_energy_wide_form_equals_tap_form(case, monkeypatch):
+    """The wide row form with 32 channels (column halves, one block per SM): dense, with cones forced on every
+    lattice (columns outside a band copied from the sample's activations, odd L, bands up to the lattice's edge), and
+    with log psi supplied, bitwise the dense tap form."""
+    name, over = case
+    w = WL[name]
+    ctx, _ = make_ctx(w, **over)
+    cfg = dev(configs_for(w, 21, seed=43, **over))
+    lp = ctx.logpsi(cfg, 'bf16')
+    got = {}
+    for key, env in (('tap', {'NQS_TC_ROWS': '0', 'NQS_TC_DENSE': '1'}), ('dense', {'NQS_TC_DENSE': '1'}),
+                     ('cones', {'NQS_TC_CONES': '1'}), ('default', {})):
+        for k, v in env.items():
+            monkeypatch.setenv(k, v)
+        got[key] = ctx.local_energy(cfg, None, 'bf16'), ctx.local_energy(cfg, lp, 'bf16')
+        for k in env:
+            monkeypatch.delenv(k)
+    ctx.sync()
+    for key in ('dense', 'cones', 'default'):
+        assert torch.equal(got[key][0], got['tap'][0]) and torch.equal(got[key][1], got['tap'][1]), key
+
+
 def test_local_energy_bf16_zero_network():
     w = WL['j1j2_10x10']
     from tests.gpu_common import problem_of
