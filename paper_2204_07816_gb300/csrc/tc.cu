@@ -2026,9 +2026,54 @@ struct TcRequest {
     int64_t n, start;   // samples, index of the first sample in the launch
 };
 
-// Local energies of several problems (same channel count) in one launch:
-// blocks take samples one at a time from a global counter in problem-major
-// order and re-bind their shared-memory plan when the problem changes.
+// Local energies of several problems through the wide row form, the requests
+// in the kernel's parameters (a plan then comes from constant memory, as in
+// the single-problem kernel: descriptors stay in uniform registers). Blocks
+// take samples one at a time from a global counter in problem-major order and
+// re-bind their shared-memory plan when the problem changes. Dense: cones pay
+// only on the largest lattices.
+constexpr int kWideGroupMax = 16;
+struct WideGroup {
+    int count;
+    TcRequest r[kWideGroupMax];
+};
+
+template <int C>
+__global__ void __launch_bounds__(kWideThreads<C>, kWideBlocks<C>)
+    eloc_wide_multi_kernel(const __grid_constant__ WideGroup grp, int64_t total, uint32_t tmem_cols,
+                           unsigned long long *counter, int *err) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ long long grab;
+    TcShared sh;
+    TcState st;
+    tc_init(sh, smem, tmem_cols, st, (blockDim.x >> 5) - kIssuers);
+    int cur = -1;
+    while (true) {
+        if (threadIdx.x == 0) grab = (long long)atomicAdd(counter, 1ull);
+        __syncthreads();
+        const int64_t g = __shfl_sync(0xffffffffu, grab, 0);
+        __syncthreads();
+        if (g >= total) break;
+        int r = 0;
+        while (r + 1 < grp.count && grp.r[r + 1].start <= g) ++r;
+        const TcRequest &q = grp.r[r];
+        if (r != cur) {
+            if (cur >= 0) tc_unbind(sh, st);
+            row_bind(q.pl, sh, q.packed, st);
+            cur = r;
+        }
+        const int64_t s = g - q.start;
+        if (!wide_sample<C>(q.pl, q.p, sh, st, q.packed, q.configs + s * q.p.N, q.logpsi ? q.logpsi + 2 * s : nullptr,
+                            q.out + 2 * s, err, nullptr))
+            break;
+    }
+    tc_fini(sh, st, tmem_cols);
+}
+
+// Local energies of several problems (same channel count) in one launch, tap
+// form: blocks take samples one at a time from a global counter in
+// problem-major order and re-bind their shared-memory plan when the problem
+// changes.
 template <int C>
 __global__ void __launch_bounds__(kTcThreads, 1) eloc_tc_multi_kernel(const TcRequest *reqs, int nreq, int64_t total,
                                                                        uint32_t tmem_cols, unsigned long long *counter,
@@ -2751,47 +2796,88 @@ int launch_eloc_tc(const Problem &p, const double *, const void *packed, const i
 
 size_t tc_multi_table_bytes(int count) { return 256 + sizeof(TcRequest) * (size_t)count; }
 
+// Each problem runs in the form its own launch would choose: those with a wide
+// plan in launches of up to kWideGroupMax problems, the others in one tap-form
+// launch. A mix of six requests (J1-J2 6x6 .. 12x12, t-J 6x6 and 12x12, both
+// channel counts, 4 layers, 512 - 2,048 samples): 11.8 ms with every problem in
+// the tap form at one block per SM, 6.6 ms this way.
 int launch_eloc_tc_multi(const TcMultiItem *items, int count, void *dev_table, int max_blocks, const LaunchEnv &env) {
     if (count <= 0) return NQS_OK;
     const int C = items[0].p.C;
-    std::vector<TcRequest> reqs((size_t)count);
-    uint32_t smem = 0, cols = 32;
-    int64_t total = 0;
+    std::vector<TcRequest> tap, wide;
     for (int i = 0; i < count; ++i) {
         const Problem &p = items[i].p;
         std::string why;
-        TcPlan pl;
-        if (p.C != C || !tc_supported(p, &why) || !best_plan(p, env.max_smem, true, 16, 1, &pl, &why)) {
+        TcRequest r;
+        if (p.C != C || !tc_supported(p, &why) || !best_plan(p, env.max_smem, true, 16, 1, &r.pl, &why)) {
             *env.msg = p.C != C ? std::string("grouped local energy needs one channel count per launch") : why;
             return NQS_ERR_UNSUPPORTED;
         }
-        reqs[i].pl = pl;
-        reqs[i].p = p;
-        reqs[i].packed = (const unsigned char *)items[i].packed;
-        reqs[i].configs = items[i].configs;
-        reqs[i].logpsi = items[i].logpsi;
-        reqs[i].out = items[i].out;
-        reqs[i].n = items[i].n;
-        reqs[i].start = total;
-        total += items[i].n;
-        smem = std::max(smem, pl.total);
-        cols = std::max(cols, pl.tmem_cols);
+        r.p = p;
+        r.packed = (const unsigned char *)items[i].packed;
+        r.configs = items[i].configs;
+        r.logpsi = items[i].logpsi;
+        r.out = items[i].out;
+        r.n = items[i].n;
+        if (r.n == 0) continue;
+        TcPlan own;
+        const bool is_wide = use_row_form(p, env.max_smem, false, &own) && own.rows == 2;
+        if (is_wide) r.pl = own;
+        (is_wide ? wide : tap).push_back(r);
     }
-    if (total == 0) return NQS_OK;
+    unsigned long long *counter = (unsigned long long *)dev_table;
+    auto reset = [&]() -> int {
+        const cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), env.stream);
+        if (e == cudaSuccess) return NQS_OK;
+        *env.msg = std::string("grouped counter: ") + cudaGetErrorString(e);
+        return NQS_ERR_CUDA;
+    };
+    const auto grid_of = [&](int64_t total, int ctas) {
+        const int64_t most = (int64_t)env.num_sms * ctas;
+        return (int)std::max<int64_t>(1, std::min(total, max_blocks > 0 ? std::min<int64_t>(max_blocks, most) : most));
+    };
+    for (size_t w0 = 0; w0 < wide.size(); w0 += kWideGroupMax) {
+        WideGroup grp{};
+        uint32_t smem = 0, cols = 32;
+        int64_t total = 0;
+        grp.count = (int)std::min<size_t>(kWideGroupMax, wide.size() - w0);
+        for (int i = 0; i < grp.count; ++i) {
+            TcRequest &r = grp.r[i] = wide[w0 + i];
+            r.start = total;
+            total += r.n;
+            smem = std::max(smem, r.pl.total);   // each plan already keeps to its blocks per SM
+            cols = std::max(cols, r.pl.tmem_cols);
+        }
+        if (int rc = reset()) return rc;
+        const int grid = grid_of(total, grp.r[0].pl.ctas), threads = 32 * (grp.r[0].pl.epi + kIssuers);
+        NQS_TC_DISPATCH(C, {
+            auto k = eloc_wide_multi_kernel<CC>;
+            if (int rc = allow_dynamic_smem(k, smem, env)) return rc;
+            k<<<grid, threads, smem, env.stream>>>(grp, total, cols, counter, env.err);
+        });
+        if (int rc = check(env, "eloc_wide_multi_kernel")) return rc;
+    }
+    if (tap.empty()) return NQS_OK;
+    uint32_t smem = 0, cols = 32;
+    int64_t total = 0;
+    for (TcRequest &r : tap) {
+        r.start = total;
+        total += r.n;
+        smem = std::max(smem, r.pl.total);
+        cols = std::max(cols, r.pl.tmem_cols);
+    }
     while (cols * (233472u / (smem + 1024u)) > 512u) smem += 1024u;
     if (smem > env.max_smem) { *env.msg = "grouped plan exceeds the shared-memory limit"; return NQS_ERR_UNSUPPORTED; }
-    unsigned long long *counter = (unsigned long long *)dev_table;
     TcRequest *dreqs = (TcRequest *)((unsigned char *)dev_table + 256);
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), env.stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(dreqs, reqs.data(), sizeof(TcRequest) * (size_t)count, cudaMemcpyHostToDevice, env.stream);
+    if (int rc = reset()) return rc;
+    const cudaError_t e =
+        cudaMemcpyAsync(dreqs, tap.data(), sizeof(TcRequest) * tap.size(), cudaMemcpyHostToDevice, env.stream);
     if (e != cudaSuccess) { *env.msg = std::string("grouped table: ") + cudaGetErrorString(e); return NQS_ERR_CUDA; }
-    const int cap = max_blocks > 0 ? std::min(max_blocks, env.num_sms) : env.num_sms;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(total, cap));
+    const int grid = grid_of(total, 1);
     NQS_TC_DISPATCH(C, {
         auto k = eloc_tc_multi_kernel<CC>;
         if (int rc = allow_dynamic_smem(k, smem, env)) return rc;
-        k<<<grid, kTcThreads, smem, env.stream>>>(dreqs, count, total, cols, counter, env.err);
+        k<<<grid, kTcThreads, smem, env.stream>>>(dreqs, (int)tap.size(), total, cols, counter, env.err);
     });
     return check(env, "eloc_tc_multi_kernel");
 }
