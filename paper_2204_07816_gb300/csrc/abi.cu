@@ -483,8 +483,8 @@ int nqs_logpsi_grad(nqs_ctx *c, const int8_t *configs, int64_t n, double *O, int
     DeviceParams dp;
     if (int rc = prepare_params(c, gp, &dp)) return rc;
     if (gp == NQS_FP32 && grad_fast_supported(c->p, c->max_smem)) {
-        const int fb = (int)std::min<int64_t>(n, (int64_t)sms_of(c) * grad_fast_blocks_per_sm(c->p));
-        if (int rc = ensure_scratch(c, grad_fast_scratch_bytes(c->p, fb))) return rc;
+        const int64_t flight = grad_fast_samples(c->p, false, n, sms_of(c), c->max_smem);
+        if (int rc = ensure_scratch(c, grad_fast_scratch_bytes(c->p, flight))) return rc;
         LaunchEnv env = env_of(c);
         return launch_grad_fast(c->p, c->params32, c->params, configs, n, O, c->scratch, c->scratch_bytes, env);
     }
@@ -512,8 +512,8 @@ int nqs_logpsi_vjp(nqs_ctx *c, const int8_t *configs, int64_t n, const double *g
     const int64_t K = vjp_chunk_samples(n), nq = (n + K - 1) / K;
     const size_t part_bytes = ((size_t)nq * c->p.P * sizeof(double) + 255) & ~(size_t)255;
     const bool fast = gp == NQS_FP32 && grad_fast_supported(c->p, c->max_smem);
-    const int blocks = (int)std::min<int64_t>(nq, (int64_t)sms_of(c) * (fast ? grad_fast_blocks_per_sm(c->p) : 2));
-    const size_t work = fast ? grad_fast_scratch_bytes(c->p, blocks) : grad_scratch_bytes(c->p, gp, blocks);
+    const size_t work = fast ? grad_fast_scratch_bytes(c->p, grad_fast_samples(c->p, true, nq, sms_of(c), c->max_smem))
+                             : grad_scratch_bytes(c->p, gp, (int)std::min<int64_t>(nq, (int64_t)sms_of(c) * 2));
     if (int rc = ensure_scratch(c, part_bytes + work)) return rc;
     LaunchEnv env = env_of(c);
     double *part = (double *)c->scratch;

@@ -70,8 +70,9 @@ int launch_grad_plain(const Problem &p, int prec, const DeviceParams &dp, const 
 size_t grad_scratch_bytes(const Problem &p, int prec, int num_blocks);
 // float32-internal backward with shared-memory working sets (grad.cu)
 bool grad_fast_supported(const Problem &p, size_t max_smem);
-int grad_fast_blocks_per_sm(const Problem &p);
-size_t grad_fast_scratch_bytes(const Problem &p, int num_blocks);
+// samples in flight (VJP: chunks) the launch would use with n of them, and the scratch they need
+int64_t grad_fast_samples(const Problem &p, bool vjp, int64_t n, int num_sms, size_t max_smem);
+size_t grad_fast_scratch_bytes(const Problem &p, int64_t samples);
 int launch_grad_fast(const Problem &p, const float *p32, const double *p64, const int8_t *configs, int64_t n,
                      double *O, void *scratch, size_t scratch_bytes, const LaunchEnv &env);
 void launch_convert_params(const double *p64, float *p32, int P, cudaStream_t s);
