@@ -15,10 +15,11 @@
 // nine taps and both outputs a thread, the 3 x 3 input window in registers),
 // so that shared-memory wavefronts stay below the FMA pipe's cycles. Bound:
 // the FMA pipe (5 dense forwards a sample) at the tiles' thread use, 78 % at
-// 10x10. Measured (GB300, 8,192 samples, 10x10, 16 channels, 6 layers):
-// GRADMS; one position and eight channels a thread, one sample a block and
-// layers of index arithmetic before: 4.89 ms. Every sum keeps its order, so
-// the results are bitwise the same.
+// 10x10. Measured (GB300, before: one position and eight channels a thread, one
+// sample a block): O of 8,192 samples, 10x10, 16 channels, 6 layers 4.88 ->
+// 3.23 ms; of 1,024 samples, 16x16, 32 channels, 8 layers 8.92 -> 4.61 ms;
+// vector-Jacobian product of 2,048 samples there 13.24 -> 6.96 ms. Every sum
+// keeps its order, so the results are bitwise the same.
 //
 // Vector-Jacobian form (VJP = true): given per-sample output gradients
 // (g_a, g_phi), one backward stream seeded with g_a w_a + g_phi w_phi gives
@@ -43,10 +44,10 @@ __host__ __device__ inline size_t a16(size_t v) { return (v + 15) & ~size_t(15);
 
 // Shared memory of a block with S samples and R backward streams.
 struct GradLayout {
-    size_t w, nbr, h, g0, g1, hbar, total;
+    size_t w, nbr, h, g0, g1, hbar, turn, total;
 };
 
-__host__ __device__ inline GradLayout grad_layout(const Problem &p, int S, int R) {
+__host__ __device__ inline GradLayout grad_layout(const Problem &p, int S, int R, bool turn) {
     const size_t act = 4 * (size_t)S * p.N * (p.C + 4);
     GradLayout g;
     size_t o = 0;
@@ -56,6 +57,8 @@ __host__ __device__ inline GradLayout grad_layout(const Problem &p, int S, int R
     g.g1 = o; o = a16(o + R * act);
     g.nbr = o; o = a16(o + 2 * (size_t)9 * S * p.N);
     g.hbar = o; o = a16(o + 4 * (size_t)S * p.C);
+    g.turn = o;   // per warp: grad_store's transposition
+    if (turn) o = a16(o + 4 * (size_t)(kGradThreads / 32) * 9 * 32);
     g.total = o;
     return g;
 }
@@ -147,17 +150,58 @@ __device__ __forceinline__ void grad_weights(const float *h, const float *g, siz
     }
 }
 
+// Nine taps of input channel c for one output channel, one value a lane in the
+// thread's registers, into nine coalesced stores: the C lanes of an output
+// channel hold 9 C consecutive parameters, turned round in shared memory (a
+// store per tap touched a sector a lane: 0.7 of 4.0 ms at 10x10).
+template <int C, typename Put>
+__device__ __forceinline__ void grad_store(float *turn, const float (&v)[9], Put put) {
+    const int lane = threadIdx.x & 31, c = lane & (C - 1);
+    if (!turn) {   // no room for the transposition
+#pragma unroll
+        for (int k = 0; k < 9; ++k) put(c * 9 + k, v[k]);
+        return;
+    }
+    float *t = turn + (lane - c) * 9;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 9; ++k) t[c * 9 + k] = v[k];
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 9; ++k) put(k * C + c, t[k * C + c]);
+}
+
+// Sums over the N sites of four channels at v (lane k takes sites k, k + 32,
+// ..., then the xor-shuffle tree); the result in every lane.
+template <int CP>
+__device__ __forceinline__ float4 grad_site_sum(const float *v, int N) {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s = threadIdx.x & 31; s < N; s += 32) {
+        const float4 x = *reinterpret_cast<const float4 *>(v + s * CP);
+        a.x += x.x, a.y += x.y, a.z += x.z, a.w += x.w;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+        a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+        a.z += __shfl_xor_sync(0xffffffffu, a.z, o);
+        a.w += __shfl_xor_sync(0xffffffffu, a.w, o);
+    }
+    return a;
+}
+
 // Backward of S samples. R: streams carried at once; VJP = false with R = 1
 // (lattices whose two streams do not fit) runs the backward once per stream.
 template <int C, int R, bool VJP>
 __device__ void grad_samples(const Problem &p, unsigned char *smem, const GradLayout &gl, const float *__restrict__ prm,
-                             const double *__restrict__ p64, int S, const int8_t *const *cfg, const GradOut<VJP> *out,
+                             const double *__restrict__ p64, int S, bool has_turn, const int8_t *const *cfg, const GradOut<VJP> *out,
                              const double *ga, const double *gp, float *Hs) {
     constexpr int CP = kConvPitch<C>, OT = 8, ST = 2, OG = C / OT;
     const int N = p.N, L = p.L, nl = p.n_layers, npos = S * N;
     float *w = reinterpret_cast<float *>(smem + gl.w), *h = reinterpret_cast<float *>(smem + gl.h);
     float *g0 = reinterpret_cast<float *>(smem + gl.g0), *g1 = reinterpret_cast<float *>(smem + gl.g1);
     float *hbar = reinterpret_cast<float *>(smem + gl.hbar);
+    float *turn = has_turn ? reinterpret_cast<float *>(smem + gl.turn) + (threadIdx.x >> 5) * 9 * 32 : nullptr;
     const uint16_t *nbr = reinterpret_cast<const uint16_t *>(smem + gl.nbr);
     float *Ss = Hs + (size_t)nl * npos * C;   // Hs, Ss: [nl][npos][C] h, sigmoid(z)
     const size_t stream = (size_t)npos * CP;  // floats between the streams of a gradient buffer
@@ -220,13 +264,10 @@ __device__ void grad_samples(const Problem &p, unsigned char *smem, const GradLa
     }
     // ---------------- head
     const float *hn = nl & 1 ? g1 : h;
-    for (int t = warp; t < S * C; t += nw) {
-        const int j = t / C, c = t - j * C;
-        float v = 0.f;
-        for (int s = lane; s < N; s += 32) v += hn[(j * N + s) * CP + c];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) hbar[t] = v;
+    for (int t = warp; t < S * (C / 4); t += nw) {
+        const int j = t / (C / 4), c = t % (C / 4) * 4;
+        const float4 v = grad_site_sum<CP>(hn + (size_t)j * N * CP + c, N);
+        if (lane == 0) *reinterpret_cast<float4 *>(hbar + j * C + c) = v;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < S * C; t += blockDim.x) {
@@ -279,16 +320,16 @@ __device__ void grad_samples(const Problem &p, unsigned char *smem, const GradLa
                     grad_weights<C, R>(h + (size_t)j * N * CP + c, gc + (size_t)j * N * CP + o, stream, L, acc);
                     const GradOut<VJP> ot = out[j];
 #pragma unroll
-                    for (int k = 0; k < 9; ++k) {
-                        const int k0 = off + (o * C + c) * 9 + k, k1 = k0 + 9 * C;
-                        if (kPasses == 2) {
-                            ot.put(k0, pass, acc[0][k].x);
-                            ot.put(k1, pass, acc[0][k].y);
-                        } else {
-                            ot.put(k0, acc[0][k].x, acc[R - 1][k].x);
-                            ot.put(k1, acc[0][k].y, acc[R - 1][k].y);
+                    for (int u = 0; u < 2; ++u)   // output channels o, o + 1
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            float v[9];
+#pragma unroll
+                            for (int k = 0; k < 9; ++k) v[k] = u ? acc[r][k].y : acc[r][k].x;
+                            grad_store<C>(turn, v, [&](int k, float x) {
+                                ot.put(off + (o + u) * C * 9 + k, kPasses == 2 ? pass : r, x);
+                            });
                         }
-                    }
                 }
             } else {
                 // one or three input channels: a thread per tap as well
@@ -310,14 +351,12 @@ __device__ void grad_samples(const Problem &p, unsigned char *smem, const GradLa
                 }
             }
             // bias gradient
-            for (int t = warp; t < R * S * C; t += nw) {
-                const int r = t / (S * C), j = t / C % S, o = t % C;
-                const float *g = gc + r * stream + (size_t)j * N * CP + o;
-                float v = 0.f;
-                for (int s = lane; s < N; s += 32) v += g[s * CP];
-#pragma unroll
-                for (int q = 16; q > 0; q >>= 1) v += __shfl_xor_sync(0xffffffffu, v, q);
-                if (lane == 0) out[j].put(off + 9 * cin * C + o, kPasses == 2 ? pass : r, v);
+            for (int t = warp; t < R * S * (C / 4); t += nw) {
+                const int r = t / (S * (C / 4)), j = t / (C / 4) % S, o = t % (C / 4) * 4;
+                const float4 v = grad_site_sum<CP>(gc + r * stream + (size_t)j * N * CP + o, N);
+                if (lane < 4)
+                    out[j].put(off + 9 * cin * C + o + lane, kPasses == 2 ? pass : r,
+                               lane < 2 ? (lane == 0 ? v.x : v.y) : (lane == 2 ? v.z : v.w));
             }
             if (l == 0) break;
             // gradient of the layer's input times silu'(z_{l-1}), into the other buffer
@@ -364,14 +403,14 @@ __device__ void grad_samples(const Problem &p, unsigned char *smem, const GradLa
 // sample at a time. grad [n][2] = (g_a, g_phi), part [ceil(n / K)][P].
 template <int C, int R, bool VJP>
 __global__ void __launch_bounds__(kGradThreads, 1)
-    grad_fast_kernel(Problem p, int S, const float *__restrict__ prm, const double *__restrict__ p64,
+    grad_fast_kernel(Problem p, int S, bool turn, const float *__restrict__ prm, const double *__restrict__ p64,
                      const int8_t *__restrict__ configs, int64_t n, double *__restrict__ O,
                      const double *__restrict__ grad, int64_t K, double *__restrict__ part, float *scratch) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ const int8_t *cfg[kGradMaxSamples];
     __shared__ GradOut<VJP> out[kGradMaxSamples];
     __shared__ double ga[kGradMaxSamples], gp[kGradMaxSamples];
-    const GradLayout gl = grad_layout(p, S, R);
+    const GradLayout gl = grad_layout(p, S, R, turn);
     conv_neighbours(reinterpret_cast<uint16_t *>(smem + gl.nbr), p.L, S);
     float *Hs = scratch + (size_t)2 * p.n_layers * S * p.N * C * blockIdx.x;
     const int64_t slots = VJP ? (n + K - 1) / K : n, steps = VJP ? K : 1;
@@ -392,34 +431,49 @@ __global__ void __launch_bounds__(kGradThreads, 1)
                 gp[threadIdx.x] = VJP ? grad[2 * sc + 1] : 0.0;
             }
             __syncthreads();
-            grad_samples<C, R, VJP>(p, smem, gl, prm, p64, S, cfg, out, ga, gp, Hs);
+            grad_samples<C, R, VJP>(p, smem, gl, prm, p64, S, turn, cfg, out, ga, gp, Hs);
         }
 }
 
-// out[k] = sum over chunks q = 0 .. nq - 1 (in order) of part[q][k].
-__global__ void vjp_reduce_kernel(const double *__restrict__ part, int64_t nq, int P, double *__restrict__ out) {
+// out[k] = sum over chunks q = 0 .. nq - 1 (in order) of part[q][k]. Sixteen
+// loads are in flight before their additions: one at a time, the loop was a
+// chain of memory latencies (product at 4x4, 1,024 chunks: 0.335 -> 0.286 ms).
+__global__ void __launch_bounds__(128) vjp_reduce_kernel(const double *__restrict__ part, int64_t nq, int P,
+                                                         double *__restrict__ out) {
+    constexpr int U = 16;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= P) return;
     double v = 0.0;
-    for (int64_t q = 0; q < nq; ++q) v += part[(size_t)q * P + k];
+    int64_t q = 0;
+    for (; q + U <= nq; q += U) {
+        double x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) x[u] = __ldcs(part + (size_t)(q + u) * P + k);
+#pragma unroll
+        for (int u = 0; u < U; ++u) v += x[u];
+    }
+    for (; q < nq; ++q) v += part[(size_t)q * P + k];
     out[k] = v;
 }
-
 
 // Streams a block carries at once, and samples S: as many as shared memory
 // holds, counted in rounds of the block's threads (a forward or input-gradient
 // tile is 72 C packed multiply-adds, a weight-gradient tile 9 N R), the
 // cheapest per sample; fewer if the call has fewer samples than SMs times S.
 int grad_streams(const Problem &p, bool vjp, size_t max_smem) {
-    return !vjp && grad_layout(p, 1, 2).total + 1024 <= max_smem ? 2 : 1;
+    return !vjp && grad_layout(p, 1, 2, false).total + 1024 <= max_smem ? 2 : 1;
 }
+
+// The transposition buffer, unless it would cost the second stream (32 channels at 16x16).
+bool grad_turn(const Problem &p, int R, size_t max_smem) { return grad_layout(p, 1, R, true).total + 1024 <= max_smem; }
 
 int grad_samples_per_block(const Problem &p, bool vjp, int64_t n, int num_sms, size_t max_smem) {
     const int R = grad_streams(p, vjp, max_smem), T = kGradThreads, OG = p.C / 8;
     const int64_t most = std::min<int64_t>(kGradMaxSamples, std::max<int64_t>(1, (n + num_sms - 1) / num_sms));
     int best = 1;
     double cost = 0.0;
-    for (int S = 1; S <= most && grad_layout(p, S, R).total + 1024 <= max_smem; ++S) {
+    const bool turn = grad_turn(p, R, max_smem);
+    for (int S = 1; S <= most && grad_layout(p, S, R, turn).total + 1024 <= max_smem; ++S) {
         const int half = (S * p.N + 1) / 2, full = R == 2 ? S * p.N : half;
         const double tiles = (OG * half + T - 1) / T + (OG * full + T - 1) / T;
         const double c = (tiles * 72.0 * p.C + (S * p.C * p.C / 2 + T - 1) / T * 9.0 * p.N * R) / S;
@@ -445,9 +499,10 @@ int launch_grad_t(const Problem &p, int S, int blocks, const float *p32, const d
                   int64_t n, double *O, const double *grad, int64_t K, double *part, float *scratch,
                   const LaunchEnv &env) {
     auto k = grad_fast_kernel<C, R, VJP>;
-    const size_t bytes = grad_layout(p, S, R).total;
+    const bool turn = grad_turn(p, R, env.max_smem);
+    const size_t bytes = grad_layout(p, S, R, turn).total;
     if (int rc = allow_dynamic_smem(k, bytes, env)) return rc;
-    k<<<blocks, kGradThreads, bytes, env.stream>>>(p, S, p32, p64, configs, n, O, grad, K, part, scratch);
+    k<<<blocks, kGradThreads, bytes, env.stream>>>(p, S, turn, p32, p64, configs, n, O, grad, K, part, scratch);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         *env.msg = std::string("grad_fast_kernel: ") + cudaGetErrorString(e);
@@ -485,7 +540,7 @@ int64_t vjp_chunk_samples(int64_t n) { return std::max<int64_t>(1, (n + 1023) / 
 
 int launch_vjp_reduce(const Problem &p, const double *part, int64_t n, double *out, const LaunchEnv &env) {
     const int64_t nq = (n + vjp_chunk_samples(n) - 1) / vjp_chunk_samples(n);
-    vjp_reduce_kernel<<<(p.P + 255) / 256, 256, 0, env.stream>>>(part, nq, p.P, out);
+    vjp_reduce_kernel<<<(p.P + 127) / 128, 128, 0, env.stream>>>(part, nq, p.P, out);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         *env.msg = std::string("vjp_reduce_kernel: ") + cudaGetErrorString(e);

@@ -81,3 +81,31 @@ def test_autograd_requires_the_context_params():
     other = ctx.params.clone().requires_grad_(True)
     with pytest.raises(ValueError):
         logpsi(other, dev(configs_for(w, 2, 1)), ctx)
+
+
+TILE_CASES = [
+    ('j1j2_10x10', {'L': 4, 'n_up': 8, 'n_down': 8, 'n_layers': 1}, 700),
+    ('j1j2_10x10', {'L': 5, 'n_up': 13, 'n_down': 12, 'n_layers': 2}, 310),
+    ('tj_12x12', {'L': 7, 'n_up': 21, 'n_down': 20, 'channels': 16, 'n_layers': 3}, 611),
+    ('j1j2_16x16', {'n_layers': 2}, 5),                                             # no room for turned stores
+    ('j1j2_16x16', {'L': 17, 'n_up': 145, 'n_down': 144, 'n_layers': 2}, 3),        # the streams one after the other
+    ('j1j2_10x10', {'L': 24, 'n_up': 288, 'n_down': 288, 'n_layers': 2}, 3),
+]
+
+
+@pytest.mark.parametrize('case', TILE_CASES, ids=lambda c: '%s-%d' % (c[0], c[1].get('L', 16)))
+def test_float32_backward_tiles_and_slots(case):
+    """The float32 backward where its tiles, a block's sample slots, the stores' transposition and the two streams
+    change: every row within 1e-4 of the float64 path, and bitwise the row of a one-sample call; the vector-Jacobian
+    product within 1e-4 of the float64 path's (both held to the oracle above)."""
+    name, over, n = case
+    w = WL[name]
+    ctx, _ = make_ctx(w, **over)
+    cfg = dev(configs_for(w, n, seed=47, **over))
+    O = ctx.logpsi_grad(cfg, 'fp32')
+    assert rel_err(O.cpu().numpy(), ctx.logpsi_grad(cfg, 'fp64').cpu().numpy()) <= 1e-4
+    for s in (0, n // 2, n - 1):
+        row = ctx.logpsi_grad(cfg[s:s + 1].contiguous(), 'fp32')
+        assert torch.equal(row[0], O[s]) and torch.equal(row[1], O[n + s])
+    g = torch.from_numpy(np.random.default_rng(48).standard_normal((n, 2))).cuda()
+    assert rel_err(ctx.logpsi_vjp(cfg, g, 'fp32').cpu().numpy(), ctx.logpsi_vjp(cfg, g, 'fp64').cpu().numpy()) <= 1e-4
