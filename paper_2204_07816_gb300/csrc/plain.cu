@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "conv_f32.cuh"
 #include "internal.h"
 #include "plain_net.cuh"
 
@@ -140,6 +141,165 @@ __global__ void __launch_bounds__(kThreads) eloc_plain_kernel(Problem p, const T
             if (!isfinite(er) || !isfinite(ei)) atomicOr(err, ERRBIT_NONFINITE);
         }
         __syncthreads();
+    }
+}
+
+// ------------------------------------------------------------------ E_loc, float32, SiLU stack
+// The float32 local energy on the register tiles of conv_f32.cuh: groups of G
+// connected configurations side by side, four positions by eight channels a
+// thread, built from the sample by their exchange instead of copied;
+// the float64 exponentials and phases of every entry are taken at the end by
+// all threads. Bound: the FMA pipe; the one-site-a-thread kernel above loaded a
+// weight for every multiply-add. Every sum and term keeps its order: bitwise
+// the same energies. Measured (GB300): 10x10, 16 channels, 6 layers, 512
+// samples 31.2 -> 7.67 ms; 7x7, 16 channels, 1,000 samples 8.75 -> 2.18;
+// 16x16 190 -> 55; 10x10, 32 channels 83.8 -> 27.4.
+constexpr int kElocF32Sites = 4;
+constexpr int kElocF32Out = 8;
+
+struct ElocF32Smem {
+    size_t a, b, w, nbr, hbar, ch, lp, scr, cum, ci, cj, sigma, total;
+};
+
+__host__ __device__ inline ElocF32Smem eloc_f32_smem(const Problem &p, int G) {
+    const size_t act = 4 * (size_t)G * p.N * (p.C + 4);
+    ElocF32Smem e;
+    size_t o = 0;
+    e.a = o; o = align16(o + act);
+    e.b = o; o = align16(o + act);
+    e.w = o; o = align16(o + 4 * (size_t)(9 * p.C * (p.C > 3 ? p.C : 3) + p.C));
+    e.hbar = o; o = align16(o + 4 * (size_t)G * p.C);
+    e.ch = o; o = align16(o + 8 * (size_t)p.n_bonds);
+    e.lp = o; o = align16(o + 16 * (size_t)(p.n_bonds + 1));
+    e.scr = o; o = align16(o + sizeof(EnumScratch));
+    e.cum = o; o = align16(o + 4 * (size_t)(p.N + 1));
+    e.nbr = o; o = align16(o + 2 * (size_t)9 * G * p.N);
+    e.ci = o; o = align16(o + 2 * (size_t)p.n_bonds);
+    e.cj = o; o = align16(o + 2 * (size_t)p.n_bonds);
+    e.sigma = o; o = align16(o + p.N);
+    e.total = o;
+    return e;
+}
+
+// One layer of the group: in -> out, [position][C + 4].
+template <int CI, int C>
+__device__ __forceinline__ void eloc_f32_layer(const float *in, float *out, const float *w, const uint16_t *nbr,
+                                               int npos, int used) {
+    constexpr int OT = kElocF32Out, ST = kElocF32Sites, CP = kConvPitch<C>, OG = C / OT;
+    const int np = (used + ST - 1) / ST;
+    const float *const src[ST] = {in, in, in, in};
+    for (int it = threadIdx.x; it < OG * np; it += blockDim.x) {
+        const int o0 = it / np * OT, q0 = it % np;
+        int q[ST];
+        float2 acc[ST][OT / 2];
+#pragma unroll
+        for (int j = 0; j < ST; ++j) {
+            q[j] = min(q0 + j * np, used - 1);
+#pragma unroll
+            for (int c = 0; c < OT / 2; ++c) acc[j][c] = *reinterpret_cast<const float2 *>(w + 9 * CI * C + o0 + 2 * c);
+        }
+        conv_accumulate<CI, C, OT, ST, false>(src, w, nbr, npos, q, o0, acc);
+#pragma unroll
+        for (int j = 0; j < ST; ++j) {
+            if (q0 + j * np >= used) continue;
+#pragma unroll
+            for (int c = 0; c < OT / 2; c += 2)
+                *reinterpret_cast<float4 *>(out + q[j] * CP + o0 + 2 * c) =
+                    make_float4(silu_f(acc[j][c].x), silu_f(acc[j][c].y), silu_f(acc[j][c + 1].x), silu_f(acc[j][c + 1].y));
+        }
+    }
+}
+
+template <int C>
+__global__ void __launch_bounds__(kThreads, 2)
+    eloc_f32_kernel(Problem p, int G, const float *__restrict__ params, const double *__restrict__ p64,
+                    const int8_t *configs, const double *logpsi, int64_t n, double *out, int *err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const ElocF32Smem es = eloc_f32_smem(p, G);
+    float *bufa = reinterpret_cast<float *>(smem + es.a), *bufb = reinterpret_cast<float *>(smem + es.b);
+    float *w = reinterpret_cast<float *>(smem + es.w), *hbar = reinterpret_cast<float *>(smem + es.hbar);
+    uint16_t *nbr = reinterpret_cast<uint16_t *>(smem + es.nbr);
+    int8_t *sigma = reinterpret_cast<int8_t *>(smem + es.sigma);
+    int16_t *ci = reinterpret_cast<int16_t *>(smem + es.ci), *cj = reinterpret_cast<int16_t *>(smem + es.cj);
+    double *ch = reinterpret_cast<double *>(smem + es.ch), *lp = reinterpret_cast<double *>(smem + es.lp);
+    int *cum = reinterpret_cast<int *>(smem + es.cum);
+    EnumScratch &scr = *reinterpret_cast<EnumScratch *>(smem + es.scr);
+    constexpr int CP = kConvPitch<C>;
+    const int N = p.N, npos = G * N, ho = head_offset(p);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int recompute = logpsi == nullptr;
+    conv_neighbours(nbr, p.L, G);
+    for (int64_t s = blockIdx.x; s < n; s += gridDim.x) {
+        __syncthreads();
+        for (int r = threadIdx.x; r < N; r += blockDim.x) sigma[r] = configs[s * N + r];
+        __syncthreads();
+        double hd;
+        const int nconn = enumerate_connected(p, sigma, ci, cj, ch, &hd, cum, scr);
+        const int n_entries = nconn + recompute;
+        for (int e0 = 0; e0 < n_entries; e0 += G) {
+            const int gc = min(G, n_entries - e0), used = gc * N;
+            for (int q = threadIdx.x; q < used; q += blockDim.x) {
+                const int g = q / N, site = q - g * N, k = e0 + g - recompute;
+                int v = sigma[site];
+                if (k >= 0) {
+                    const int i = ci[k], j = cj[k];
+                    if (!NQS_INDEX_OK(k < nconn && i >= 0 && i < N && j >= 0 && j < N, err)) v = 0;
+                    else if (site == i) v = sigma[j];
+                    else if (site == j) v = sigma[i];
+                }
+                *reinterpret_cast<float4 *>(bufa + q * CP) =
+                    p.c_in == 1 ? make_float4((float)v, 0.f, 0.f, 0.f)
+                                : make_float4((float)(v == 0), (float)(v == 1), (float)(v == -1), 0.f);
+            }
+            float *in = bufa, *o = bufb;
+            for (int l = 0; l < p.n_layers; ++l) {
+                const int cin = layer_cin(p, l);
+                conv_stage<C, false>(params + layer_offset(p, l), cin, w);
+                __syncthreads();
+                if (l > 0) eloc_f32_layer<C, C>(in, o, w, nbr, npos, used);
+                else if (cin == 1) eloc_f32_layer<1, C>(in, o, w, nbr, npos, used);
+                else eloc_f32_layer<3, C>(in, o, w, nbr, npos, used);
+                __syncthreads();
+                float *t = in;
+                in = o;
+                o = t;
+            }
+            // head: sums over sites per (configuration, channel), then float64
+            for (int t = warp; t < gc * C; t += nw) {
+                const int g = t / C, c = t - g * C;
+                float v = 0.f;
+                for (int q = lane; q < N; q += 32) v += in[(g * N + q) * CP + c];
+#pragma unroll
+                for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
+                if (lane == 0) hbar[t] = v;
+            }
+            __syncthreads();
+            for (int t = threadIdx.x; t < 2 * gc; t += blockDim.x) {
+                const int g = t >> 1, out_k = t & 1;
+                double sum = 0.0;
+                for (int c = 0; c < C; ++c) sum = fma(p64[ho + out_k * C + c], (double)hbar[g * C + c], sum);
+                lp[2 * (e0 + g) + out_k] = sum;
+            }
+        }
+        __syncthreads();
+        const double a0 = recompute ? lp[0] : logpsi[2 * s], phi0 = recompute ? lp[1] : logpsi[2 * s + 1];
+        __syncthreads();
+        for (int k = threadIdx.x; k < nconn; k += blockDim.x) {
+            double *e = lp + 2 * (k + recompute);
+            const double m = ch[k] * exp(e[0] - a0);
+            double sn, cs;
+            sincos(e[1] - phi0, &sn, &cs);
+            e[0] = m * cs;
+            e[1] = m * sn;
+        }
+        __syncthreads();
+        if (lane == 0 && warp < 2) {   // terms added in list order: real parts by one warp, imaginary by another
+            double sum = 0.0;
+            for (int k = 0; k < nconn; ++k) sum += lp[2 * (k + recompute) + warp];
+            const double v = warp == 0 ? hd + sum : sum;
+            out[2 * s + warp] = v;
+            if (!isfinite(v)) atomicOr(err, ERRBIT_NONFINITE);
+        }
     }
 }
 
@@ -561,6 +721,40 @@ int launch_logpsi_plain(const Problem &p, int prec, const DeviceParams &dp, cons
     return logpsi_plain_t<float>(p, dp.p32, dp.p64, configs, n, out, env);
 }
 
+// Group size of the float32 kernel: the most useful threads per round of the
+// block's tiles with two blocks per SM (one if a configuration needs more);
+// 0 if no group fits.
+static int eloc_f32_group(const Problem &p, size_t max_smem) {
+    const int OG = p.C / kElocF32Out;
+    int best = 0;
+    double score = 0.0;
+    for (size_t cap : {std::min<size_t>(max_smem, 233472 / 2 - 1024), max_smem}) {
+        for (int G = 1; G <= 32 && (size_t)G * p.N <= 8192 && eloc_f32_smem(p, G).total <= cap; ++G) {
+            const int tiles = OG * ((G * p.N + kElocF32Sites - 1) / kElocF32Sites);
+            const double sc = (double)(OG * G * p.N) / ((tiles + kThreads - 1) / kThreads);
+            if (sc > score + 1e-9) { score = sc; best = G; }
+        }
+        if (best) return best;
+    }
+    return 0;
+}
+
+static int eloc_f32(const Problem &p, int G, const float *params, const double *p64, const int8_t *configs,
+                    const double *logpsi, int64_t n, double *out, const LaunchEnv &env) {
+    const size_t bytes = eloc_f32_smem(p, G).total;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)env.num_sms * 2));
+    auto go = [&](auto k) {
+        if (int rc = set_smem<float>(k, bytes, env)) return rc;
+        k<<<grid, kThreads, bytes, env.stream>>>(p, G, params, p64, configs, logpsi, n, out, env.err);
+        return check_launch(env, "eloc_f32_kernel");
+    };
+    switch (p.C) {
+        case 8: return go(eloc_f32_kernel<8>);
+        case 16: return go(eloc_f32_kernel<16>);
+        default: return go(eloc_f32_kernel<32>);
+    }
+}
+
 template <typename T>
 static int eloc_plain_t(const Problem &p, const T *params, const double *p64, const int8_t *configs,
                         const double *logpsi, int64_t n, double *out, const LaunchEnv &env) {
@@ -582,6 +776,11 @@ int launch_eloc_plain(const Problem &p, int prec, const DeviceParams &dp, const 
                       const double *logpsi, int64_t n, double *out, const LaunchEnv &env) {
     if (n == 0) return NQS_OK;
     if (prec == NQS_FP64) return eloc_plain_t<double>(p, dp.p64, dp.p64, configs, logpsi, n, out, env);
+    // the paper's families, four channels (a 4x4 batch of 1,000 samples: 0.099 ms in tiles, 0.078 in the general
+    // kernel's eight blocks per SM) and lattices whose activations do not fit the tiles' pitch keep the general kernel
+    if (p.net == NQS_NET_SILU && p.C >= 8)
+        if (const int G = eloc_f32_group(p, env.max_smem))
+            return eloc_f32(p, G, dp.p32, dp.p64, configs, logpsi, n, out, env);
     return eloc_plain_t<float>(p, dp.p32, dp.p64, configs, logpsi, n, out, env);
 }
 

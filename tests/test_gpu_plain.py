@@ -127,6 +127,32 @@ def test_local_energy_fp32_energy_per_site():
     assert rel_err(got[:, 0], want.real) <= 1e-4
 
 
+@pytest.mark.parametrize('name,over,n', [
+    ('j1j2_10x10', {'L': 4, 'n_up': 8, 'n_down': 8, 'channels': 8, 'n_layers': 1}, 40),
+    ('j1j2_10x10', {'L': 5, 'n_up': 13, 'n_down': 12, 'channels': 8, 'n_layers': 3}, 40),
+    ('j1j2_10x10', {'L': 7, 'n_up': 25, 'n_down': 24, 'n_layers': 2}, 30),
+    ('tj_12x12', {'n_layers': 2}, 12),
+    ('tj_12x12', {'L': 6, 'n_up': 1, 'n_down': 1, 'channels': 16, 'n_layers': 2}, 20),
+    ('j1j2_16x16', {'n_layers': 2}, 6),
+])
+@pytest.mark.parametrize('give_logpsi', [False, True])
+def test_local_energy_fp32_tiles(name, over, n, give_logpsi):
+    """The float32 local energy's register tiles over channel counts, odd lattices, a last group of few configurations
+    and both inputs: within 1e-5 per site of the float64 path on every sample (log psi differences carry float32
+    rounding of O(N C) terms, about 1e-6 here), and the rows of a smaller batch bitwise the same."""
+    w = WL[name]
+    ctx, _ = make_ctx(w, **over)
+    N = over.get('L', w['L']) ** 2
+    cfg = dev(configs_for(w, n, seed=61, **over))
+    lp = ctx.logpsi(cfg, 'fp32') if give_logpsi else None
+    got = ctx.local_energy(cfg, lp, 'fp32')
+    want = ctx.local_energy(cfg, None, 'fp64')
+    assert float((got - want).abs().max()) / N <= 1e-5
+    k = n // 2
+    part = ctx.local_energy(cfg[k:].contiguous(), lp[k:].contiguous() if give_logpsi else None, 'fp32')
+    assert torch.equal(part, got[k:])
+
+
 def test_zero_network_closed_form_on_gpu():
     """All parameters zero: E_loc = (J1 + J2) N / 2 for every configuration."""
     w = WL['j1j2_10x10']
