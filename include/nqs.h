@@ -127,7 +127,8 @@ int64_t nqs_param_count(const nqs_problem *p);
  * opt-in shared memory per block (host only, no GPU work; the launchers use
  * the same code with the current device's values). kind: 0 = nqs_logpsi,
  * 1 = nqs_local_energy (n = samples), 2 = nqs_sample (n = chains).
- * out: host int32 [9] = configurations per group (G), groups in flight per
+ * out: host int32 [9] = configurations per group (G; kind 2: chains per
+ * group, whose next proposals may be evaluated ahead), groups in flight per
  * block, blocks per SM the plan is sized for, epilogue warps, 128-row tiles
  * per group, shared-memory bytes per block, tensor-memory columns per block,
  * grid size, form (0: one MMA per 3x3 tap and 128-row tile of padded

@@ -56,6 +56,7 @@ constexpr int kTcThreads = 32 * (kMaxEpiWarps + kIssuers);
 // sampler is compiled for two blocks at both widths.
 template <int C> constexpr int kMinBlocks = C == 16 ? 2 : 1;
 constexpr int kMaxTiles = 16;
+constexpr int kMaxAhead = 4;     // sampler: proposals of one chain evaluated together, at most
 constexpr int kPropWindow = 16;   // sampler: proposal steps drawn at once
 constexpr int kPropWindowOne = 64;   // the same with one chain per block (one draw per thread either way)
 __host__ __device__ inline int prop_window(int per_block) { return per_block == 1 ? kPropWindowOne : kPropWindow; }
@@ -2117,9 +2118,151 @@ __device__ __forceinline__ int neighbour_dir_tc(int i, int d, int L) {
     return ((y + dy + L) % L) * L + (x + dx + L) % L;
 }
 
-// Metropolis exchange sampler. Each block owns up to slots * G chains;
-// slot s evaluates the proposals of chains s * G ... s * G + G - 1.
+// One sweep of one chain, proposals evaluated ahead. The proposals do not
+// depend on the chain's state, so the group's G configurations are the next
+// proposals that change the state, each on the state that follows if the ones
+// before it end as predicted: accepted if log u < `typical`, a running centre
+// of 2 (a' - a). They are then decided in order, each against the true current
+// amplitude; at the first outcome that differs from its prediction the rest is
+// dropped and evaluated again on the true state. So the chain, its log psi and
+// its counters are those of one proposal at a time, whatever is predicted. A
+// forward of one configuration is a chain of latencies that leaves the SM
+// mostly idle (one tile of MMAs per layer), and further configurations cost
+// little beside it. Measured (GB300, ms for four sweeps, one proposal at a time
+// / ahead): 10x10, 16 channels, 6 layers: 152 chains 1.55 / 0.84 at an
+// acceptance of 1.0, 1.51 / 1.01 at 0.9, 1.49 / 1.16 at 0.13; 256 chains 1.71 /
+// 1.20, 1.68 / 1.34, 1.63 / 1.48; 1,024 chains 4.86 / 3.31, 4.84 / 3.62, 4.68 /
+// 4.15. t-J 12x12, 32 channels, 256 chains, 0.53: 6.10 / 5.07. 16x16, 32
+// channels, 8 layers, 128 chains: 12.6 / 5.6.
+// Every thread follows the state (the last block barrier followed its update)
+// and every warp picks the proposals by itself, its lanes over the next 32.
 template <int C>
+__device__ bool sample_ahead(const TcPlan &pl, const TcShared &sh, const unsigned char *packed, TcState &st, int *err,
+                             int8_t *cur, int *wpi, int *wpj, double *wlu, int W, int64_t &wbase, float *typical,
+                             int *advance, double *ca, double *cphi, unsigned long long *counts, int64_t first,
+                             int64_t n_steps, uint64_t chain, uint64_t step0, uint64_t seed) {
+    const int G = pl.G, N = pl.N, lane = threadIdx.x & 31;
+    int q = 0;   // next proposal of the sweep
+    while (q < N) {
+        const int64_t gstep = first + q;
+        if (gstep >= wbase + W) {   // draw the next window (one Philox4x64-10 block per step)
+            __syncthreads();        // every thread is done with the previous one
+            wbase = gstep;
+            for (int t = threadIdx.x; t < W; t += blockDim.x) {
+                if (gstep + t >= n_steps) continue;
+                const Philox4 b = philox(chain, step0 + (uint64_t)(gstep + t), 0, 0, seed, 0);
+                const int i = (int)mulhi64(b.v[0], (uint64_t)N);
+                wpi[t] = i;
+                wpj[t] = neighbour_dir_tc(i, (int)(b.v[1] >> 62), pl.L);
+                const double u = (double)(b.v[2] >> 11) * 0x1.0p-53;
+                wlu[t] = u > 0.0 ? log(u) : -INFINITY;
+            }
+            __syncthreads();
+        }
+        const int at = (int)(gstep - wbase), avail = min(min(W - at, N - q), 32);
+        // this lane's proposal, the values of its two sites on the predicted state and its own prediction
+        int pi = 0, pj = 0, vi = 0, vj = 0;
+        uint32_t accept = 0u;
+        if (lane < avail) {
+            pi = wpi[at + lane];
+            pj = wpj[at + lane];
+            accept = (float)wlu[at + lane] < *typical;
+            if (NQS_INDEX_OK(pi >= 0 && pi < N && pj >= 0 && pj < N, err)) { vi = cur[pi]; vj = cur[pj]; }
+        }
+        uint32_t moves = __ballot_sync(0xffffffffu, vi != vj);
+        if (!moves) { q += avail; continue; }
+        // pick up to G moves (sites below 2,048, values + 1 in two bits)
+        int m = 0, off[kMaxAhead], si[kMaxAhead], sj[kMaxAhead], a_i[kMaxAhead], a_j[kMaxAhead];
+        uint32_t pred = 0u;   // bit k: move k predicted accepted
+#pragma unroll
+        for (int k = 0; k < kMaxAhead; ++k) {
+            off[k] = 0, si[k] = sj[k] = -1, a_i[k] = a_j[k] = 0;
+            if (k < G && moves) {
+                const int f = __ffs(moves) - 1;
+                const uint32_t w = __shfl_sync(0xffffffffu, (uint32_t)pi | (uint32_t)pj << 11 | (uint32_t)(vi + 1) << 22 |
+                                                                (uint32_t)(vj + 1) << 24 | accept << 26, f);
+                off[k] = f;
+                si[k] = (int)(w & 2047u);
+                sj[k] = (int)(w >> 11 & 2047u);
+                a_i[k] = (int)(w >> 22 & 3u) - 1;
+                a_j[k] = (int)(w >> 24 & 3u) - 1;
+                if (w >> 26) {   // the two sites' values exchanged from here on
+                    pred |= 1u << k;
+                    vi = pi == si[k] ? a_j[k] : (pi == sj[k] ? a_i[k] : vi);
+                    vj = pj == si[k] ? a_j[k] : (pj == sj[k] ? a_i[k] : vj);
+                    moves = __ballot_sync(0xffffffffu, vi != vj);
+                }
+                moves &= ~((2u << f) - 1u);
+                ++m;
+            }
+        }
+        for (int s = threadIdx.x; s < N; s += blockDim.x) {
+            int v = cur[s];
+#pragma unroll
+            for (int k = 0; k < kMaxAhead; ++k) {
+                if (k >= G) break;
+                const int x = s == si[k] ? a_j[k] : (s == sj[k] ? a_i[k] : v);   // unused slots: the state itself
+                sh.spins[k * N + s] = (int8_t)x;
+                if (pred >> k & 1u) v = x;
+            }
+        }
+        __syncthreads();
+        if (!tc_forward<C>(pl, sh, packed, st, err)) return false;
+        if (threadIdx.x < 32) {
+            // lane k decides move k as if the moves before it went as predicted; the first that did not is the last
+            // that counts
+            double delta = 0.0;
+            bool acc = false;
+            if (lane < m) {
+                const uint32_t before = pred & ((1u << lane) - 1u);
+                const double base = before ? sh.res[31 - __clz(before)] : ca[0];
+                int o = off[0];
+#pragma unroll
+                for (int k = 1; k < kMaxAhead; ++k) o = lane == k ? off[k] : o;
+                delta = 2.0 * (sh.res[lane] - base);
+                // u < exp(2 (a' - a)) evaluated as log u < 2 (a' - a), log u drawn with the proposal
+                acc = delta >= 0.0 || wlu[at + o] < delta;
+            }
+            const uint32_t accepted = __ballot_sync(0xffffffffu, acc);
+            const uint32_t wrong = (accepted ^ pred) & ((1u << m) - 1u);
+            const int last = wrong ? __ffs(wrong) - 1 : m - 1;
+            const uint32_t took = accepted & ((2u << last) - 1u);
+            float pull = lane <= last ? fminf(fmaxf((float)delta - *typical, -0.2f), 0.2f) : 0.f;
+#pragma unroll
+            for (int o = 1; o < kMaxAhead; o <<= 1) pull += __shfl_xor_sync(0xffffffffu, pull, o);
+            if (lane == 0) {
+                int adv = avail;   // every prediction right, fewer than G moves: none is left among these proposals
+#pragma unroll
+                for (int k = 0; k < kMaxAhead; ++k) {
+                    if (took >> k & 1u) {
+                        cur[si[k]] = (int8_t)a_j[k];
+                        cur[sj[k]] = (int8_t)a_i[k];
+                    }
+                    if (k == last && (wrong || m == G)) adv = off[k] + 1;
+                }
+                if (took) {
+                    const int k = 31 - __clz(took);
+                    ca[0] = sh.res[k];
+                    cphi[0] = sh.res[G + k];
+                }
+                counts[0] += (unsigned long long)(last + 1);
+                counts[1] += (unsigned long long)__popc(took);
+                *typical += 0.25f * pull;
+                *advance = adv;
+            }
+        }
+        __syncthreads();
+        const int adv = *advance;
+        q += adv;
+    }
+    return true;
+}
+
+// Metropolis exchange sampler. Each block owns up to slots * G chains; slot s
+// evaluates the proposals of chains s * G ... s * G + G - 1. AHEAD (one chain a
+// block): the group's configurations are proposals of that chain
+// (sample_ahead).
+template <int C, bool AHEAD>
 __global__ void __launch_bounds__(kTcThreads, 2) sample_tc_kernel(TcPlan pl, const unsigned char *packed,
                                                                    int8_t *chains, int n_chains, int per_block,
                                                                    uint64_t step0, uint64_t seed, int spc,
@@ -2161,7 +2304,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) sample_tc_kernel(TcPlan pl, con
     {
         for (int r = threadIdx.x; r < gc * N; r += blockDim.x) cur[r] = chains[(size_t)c0 * N + r];
         __syncthreads();
-        for (int r = threadIdx.x; r < per_block * N; r += blockDim.x) {
+        for (int r = threadIdx.x; r < G * S * N; r += blockDim.x) {
             const int c = r / N;
             sh.spins[r] = cur[(c < gc ? c : 0) * N + (r - c * N)];
         }
@@ -2176,8 +2319,23 @@ __global__ void __launch_bounds__(kTcThreads, 2) sample_tc_kernel(TcPlan pl, con
     }
     const int n_sweeps = burn_in + spc * sweeps_between;
     const int64_t n_steps = (int64_t)n_sweeps * N;
+    // AHEAD: step of the window's first proposal; in shared memory, 2 (a' - a) of a typical move and the proposals
+    // decided by the last forward
+    int64_t wbase = -W;
+    float *typical = reinterpret_cast<float *>(list2);
+    int *advance = list2 + 1;
+    if (AHEAD) {
+        if (threadIdx.x == 0) *typical = 0.f;
+        __syncthreads();
+    }
     for (int sweep = 0; ok && sweep < n_sweeps; ++sweep) {
-        for (int q = 0; q < N; ++q) {
+        if constexpr (AHEAD) {
+            ok = sample_ahead<C>(pl, sh, packed, st, err, cur, wpi, wpj, wlu, W, wbase, typical, advance, ca, cphi,
+                                 scnt(),
+                                 (int64_t)sweep * N, n_steps, (uint64_t)c0, step0, seed);
+            if (!ok) break;
+        }
+        for (int q = 0; !AHEAD && q < N; ++q) {
             const int64_t gstep = (int64_t)sweep * N + q;
             const int w = (int)(gstep & (int64_t)(W - 1));
             if (w == 0) {   // draw the window (one Philox4x64-10 block per chain and step)
@@ -2579,8 +2737,8 @@ int eloc_extra(const Problem &p) {
                  4 * sizeof(double) + 16 * (chunk + 1) + 8 * 258 + 2 * ((chunk + 1) & ~1) + 4 * 32);
 }
 
-int sample_extra(const Problem &p, int G, int slots) {
-    const int per = G * slots;
+// per: chains of a block
+int sample_extra(const Problem &p, int G, int slots, int per) {
     return (int)(al16(per * p.N) + al16(4 * 2 * (slots * (G + 1))) + 16 * per + 16 * prop_window(per) * per + 24);
 }
 
@@ -2895,30 +3053,55 @@ namespace {
 // earlier plans of 3 to 10 chains per block at one block per SM (the chains
 // are the same bit for bit: a configuration's log psi does not depend on its
 // row in the tile).
-bool sample_plan(const Problem &p, size_t max_smem, TcPlan *out, std::string *why) {
+bool sample_plan(const Problem &p, size_t max_smem, int64_t n_chains, int num_sms, TcPlan *out, int *per_block,
+                 std::string *why) {
     int fg = 0, fs = 0, fc = 1;
     const char *force = getenv("NQS_TC_SAMPLE");   // "G,slots,blocks per SM" (tuning)
     const bool forced = force && sscanf(force, "%d,%d,%d", &fg, &fs, &fc) == 3 && fc >= 1 && fc <= 3 && fg >= 1;
     if (!forced) {
+        *per_block = 1;
         // the kernel is compiled for two blocks of kTcThreads threads, so it uses at most 96 registers a thread
         // (65,536 / 640, in steps of 8); a launch of fewer threads leaves room for a third block
         constexpr int kRegsCap = 65536 / (2 * kTcThreads) / 8 * 8;
-        for (int ctas = 3; ctas >= 1; --ctas)
-            if (make_plan(p, 1, 1, ctas, max_smem, sample_extra(p, 1, 1), out, why)) {
+        bool found = false;
+        for (int ctas = 3; ctas >= 1 && !found; --ctas)
+            if (make_plan(p, 1, 1, ctas, max_smem, sample_extra(p, 1, 1, 1), out, why)) {
                 // one epilogue warp per TMEM lane quarter (measured 8 % faster than eight warps)
                 if (out->n_tiles <= 4) out->epi = 4;
-                if (ctas * 32 * (out->epi + kIssuers) * kRegsCap > 65536) continue;
-                return true;
+                found = ctas * 32 * (out->epi + kIssuers) * kRegsCap <= 65536;
             }
-        return false;
+        if (!found) return false;
+        // Proposals evaluated ahead (sample_ahead): four with one block per SM, three with more (two with three blocks of
+        // 32 channels), fewer where the blocks
+        // per SM that this many chains can use would not fit (one block less costs more than a poor prediction gains
+        // back: 16x16, 32 channels, 304 chains with an acceptance of 0.15 14.5 -> 15.3 ms, of 1.0 14.3 -> 11.5). Eight
+        // epilogue warps with one block per SM, and with two where a tile has 32 channels.
+        const int need = (int)std::min<int64_t>(out->ctas, (n_chains + num_sms - 1) / num_sms);
+        const char *ahead = getenv("NQS_TC_AHEAD");   // tuning
+        const int most = ahead ? std::min(atoi(ahead), kMaxAhead) : (need == 1 ? 4 : (need == 3 && p.C == 32 ? 2 : 3));
+        const int epi = need == 1 || (need == 2 && p.C == 32) ? 8 : 4;
+        for (int D = most; D > 1; --D) {
+            TcPlan pl;
+            std::string w;
+            // the plan's own blocks per SM if eight epilogue warps leave the registers, else two or what is needed
+            const int first = epi == 8 ? std::min(out->ctas, 2) : out->ctas;
+            if (!make_plan(p, D, 1, first, max_smem, sample_extra(p, D, 1, 1), &pl, &w) &&
+                !make_plan(p, D, 1, need, max_smem, sample_extra(p, D, 1, 1), &pl, &w))
+                continue;
+            pl.epi = epi;
+            *out = pl;
+            break;
+        }
+        return true;
     }
     for (int ctas = fc; ctas >= 1; --ctas) {   // fewer blocks per SM if the forced count does not fit
         const int slots = std::min(std::max(fs, 1), kMaxSlots);
         for (int G = std::min(fg, 16); G >= 1; --G)
-            if (make_plan(p, G, slots, ctas, max_smem, sample_extra(p, G, slots), out, why)) {
+            if (make_plan(p, G, slots, ctas, max_smem, sample_extra(p, G, slots, G * slots), out, why)) {
                 // a sampler group is one or a few tiles: one epilogue warp per
                 // TMEM lane quarter (measured 8 % faster than eight warps)
                 if (out->slots * out->n_tiles <= 4) out->epi = 4;
+                *per_block = out->G * out->slots;
                 return true;
             }
     }
@@ -2928,8 +3111,8 @@ bool sample_plan(const Problem &p, size_t max_smem, TcPlan *out, std::string *wh
 // Sampler grid: one block per chain group, or, when the groups outnumber the
 // co-resident blocks and a group holds several chains or the context is held
 // to an SM share, the co-resident blocks, each taking several groups in turn.
-int64_t sample_grid(const TcPlan &pl, int64_t n_chains, int num_sms, bool sm_limited) {
-    const int64_t per = (int64_t)pl.G * pl.slots, groups = (n_chains + per - 1) / per;
+int64_t sample_grid(const TcPlan &pl, int64_t per, int64_t n_chains, int num_sms, bool sm_limited) {
+    const int64_t groups = (n_chains + per - 1) / per;
     if (per == 1 && !sm_limited) return groups;
     return std::min<int64_t>(groups, (int64_t)num_sms * pl.ctas);
 }
@@ -2941,14 +3124,14 @@ int launch_sample_tc(const Problem &p, const double *, const void *packed, int8_
                      double *out_logpsi, const LaunchEnv &env) {
     std::string why;
     TcPlan pl;
-    if (!tc_supported(p, &why) || !sample_plan(p, env.max_smem, &pl, &why)) {
+    int per_block = 1;
+    if (!tc_supported(p, &why) || !sample_plan(p, env.max_smem, n_chains, env.num_sms, &pl, &per_block, &why)) {
         *env.msg = why;
         return NQS_ERR_UNSUPPORTED;
     }
-    const int per_block = pl.G * pl.slots;
-    const int grid = (int)sample_grid(pl, n_chains, env.num_sms, env.sm_limited);
+    const int grid = (int)sample_grid(pl, per_block, n_chains, env.num_sms, env.sm_limited);
     NQS_TC_DISPATCH(p.C, {
-        auto k = sample_tc_kernel<CC>;
+        auto k = per_block == 1 && pl.G > 1 ? sample_tc_kernel<CC, true> : sample_tc_kernel<CC, false>;
         if (int rc = prep(k, pl, env)) return rc;
         k<<<grid, 32 * (pl.epi + kIssuers), pl.total, env.stream>>>(pl, (const unsigned char *)packed, chains,
                                                                     n_chains, per_block, step0, seed, spc,
@@ -2966,19 +3149,20 @@ int launch_wait_probe(int64_t iterations, const LaunchEnv &env) {
 int tc_describe_plan(const Problem &p, int kind, int64_t n, size_t max_smem, int num_sms, int32_t *out,
                      std::string *why) {
     TcPlan pl;
+    int per_block = 1;
     bool ok = tc_supported(p, why);
     if (ok) {
-        if (kind == 2) ok = sample_plan(p, max_smem, &pl, why);
+        if (kind == 2) ok = sample_plan(p, max_smem, n, num_sms, &pl, &per_block, why);
         else if (kind == 1 && use_row_form(p, max_smem, false, &pl)) ok = true;
         else ok = best_plan(p, max_smem, kind == 1, 16, 2, &pl, why);
     }
     if (!ok) return NQS_ERR_UNSUPPORTED;
     const int64_t per = (int64_t)pl.G * pl.slots, cap = (int64_t)num_sms * pl.ctas;
     int64_t grid;
-    if (kind == 2) grid = sample_grid(pl, n, num_sms, false);
+    if (kind == 2) grid = sample_grid(pl, per_block, n, num_sms, false);
     else if (kind == 1) grid = std::max<int64_t>(1, std::min<int64_t>(n, cap));
     else grid = std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, cap));
-    out[0] = pl.G;
+    out[0] = kind == 2 ? per_block / pl.slots : pl.G;   // sampler: chains per group
     out[1] = pl.slots;
     out[2] = pl.ctas;
     out[3] = pl.epi;

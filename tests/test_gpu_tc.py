@@ -362,6 +362,44 @@ def test_sampler_bf16_waves_of_chains():
     assert torch.equal(ctx_a.logpsi(cfg_a, 'bf16'), lp_a)
 
 
+AHEAD_CASES = [
+    ('j1j2_10x10', {}, 256, 0.5),
+    ('j1j2_10x10', {}, 40, 1.5),
+    ('j1j2_4x4', {'channels': 16, 'n_layers': 2}, 700, 1.5),      # sweeps of 16 proposals
+    ('j1j2_10x10', {'L': 5, 'n_up': 13, 'n_down': 12, 'n_layers': 3}, 330, 1.0),
+    ('tj_12x12', {}, 160, 1.5),
+    ('tj_12x12', {'L': 6, 'n_up': 1, 'n_down': 0, 'channels': 16, 'n_layers': 2}, 9, 2.0),   # most proposals move nothing
+    ('j1j2_16x16', {'n_layers': 3}, 24, 1.0),
+]
+
+
+@pytest.mark.parametrize('case', AHEAD_CASES, ids=lambda c: '%s-%d-%d' % (c[0], c[1].get('L', 0), c[2]))
+def test_sampler_ahead_equals_one_proposal_at_a_time(case, monkeypatch):
+    """Proposals evaluated ahead on predicted states and decided in order give bitwise the chains, log psi and move
+    counters of one proposal at a time, whatever was predicted (acceptances from 0.1 to 1.0), over several calls,
+    sweeps that end inside a window and chains that share an SM."""
+    name, over, chains, scale = case
+    w = WL[name]
+    runs = []
+    for ahead in ('1', None, '2', '3'):
+        if ahead:
+            monkeypatch.setenv('NQS_TC_AHEAD', ahead)
+        ctx, _ = make_ctx(w, seed=19, scale=scale, **over)
+        a = ctx.sample(chains, 2, 1, 1, 'bf16')
+        if ahead == '2':
+            ctx.set_sm_limit(10)
+        b = ctx.sample(chains, 1, 2, 0, 'bf16')
+        runs.append((a, b, ctx.sampler_counts(), ctx.get_chains(chains)))
+        ctx.sync()
+        if ahead:
+            monkeypatch.delenv('NQS_TC_AHEAD')
+    (a0, b0, n0, c0) = runs[0]
+    for a, b, n, c in runs[1:]:
+        for x, y in ((a, a0), (b, b0)):
+            assert torch.equal(x[0], y[0]) and torch.equal(x[1], y[1])
+        assert n == n0 and c[1] == c0[1] and torch.equal(c[0], c0[0])
+
+
 def nqs_param_count_of(w, **over):
     from tests.gpu_common import problem_of
     return lib().nqs_param_count(problem_of(w, **over))
