@@ -138,7 +138,7 @@ int prepare_params(nqs_ctx *c, int prec, DeviceParams *dp) {
         ++c->launches;
     } else if (prec == NQS_BF16 || prec == NQS_FP8) {
         LaunchEnv env = env_of(c);
-        int rc = launch_tc_pack(c->p, c->params, c->packed, env);
+        int rc = launch_tc_pack(c->p, c->params, c->packed, prec == NQS_FP8, env);
         if (rc) return rc;
     }
     return NQS_OK;
@@ -328,7 +328,7 @@ int nqs_local_energy_multi(nqs_ctx *const *ctxs, int32_t count, const int8_t *co
         for (int i = 0; i < count; ++i) {
             nqs_ctx *c = ctxs[i];
             if (c->p.C != C) continue;
-            if (int rc = launch_tc_pack(c->p, c->params, c->packed, env)) return rc;
+            if (int rc = launch_tc_pack(c->p, c->params, c->packed, false, env)) return rc;
             TcMultiItem it;
             it.p = c->p;
             it.packed = c->packed;

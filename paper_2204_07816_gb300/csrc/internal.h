@@ -89,7 +89,8 @@ int launch_vjp_reduce(const Problem &p, const double *part, int64_t n, double *o
 // ---- tensor-core path (tc.cu)
 bool tc_supported(const Problem &p, std::string *why);
 size_t tc_packed_bytes(const Problem &p);
-int launch_tc_pack(const Problem &p, const double *p64, void *packed, const LaunchEnv &env);
+// f8: the e4m3 images too (read by the FP8 local energies only)
+int launch_tc_pack(const Problem &p, const double *p64, void *packed, bool f8, const LaunchEnv &env);
 int launch_logpsi_tc(const Problem &p, const double *p64, const void *packed, const int8_t *configs, int64_t n,
                      double *out, const LaunchEnv &env);
 size_t tc_eloc_cache_bytes(const Problem &p, size_t max_smem, int num_sms, int64_t n);

@@ -2459,7 +2459,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) sample_tc_kernel(TcPlan pl, con
 // zero for k >= 9 c_in. bf16 block per layer l >= 1: [9][C / 8][C][8],
 // element (tap o, k = c_in, n = c_out); then the same layers again in the
 // row form's order [3][C / 8][3][C][8].
-__global__ void tc_pack_kernel(Problem p, TcPlan pl, const double *params, unsigned char *packed) {
+__global__ void tc_pack_kernel(Problem p, TcPlan pl, const double *params, unsigned char *packed, bool f8) {
     const int C = p.C;
     float *f = reinterpret_cast<float *>(packed);
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
@@ -2493,31 +2493,32 @@ __global__ void tc_pack_kernel(Problem p, TcPlan pl, const double *params, unsig
         const int dyi = o / 3, j = 2 - o % 3;
         dr[(((dyi * (C / 8) + k / 8) * 3 + j) * C + n) * 8 + (k % 8)] = __float2bfloat16_rn((float)w);
     }
-    // e4m3 images of layers >= 1 (layer 0 keeps bf16 operands); the scale of output channel n is the largest
-    // |weight| of the channel over 448, the largest e4m3 value
-    if (pl.f8bytes == 0) return;
-    for (int e = tid; e < (p.n_layers - 1) * C; e += nth) {
+    // e4m3 images of layers >= 1 (layer 0 keeps bf16 operands), for the calls that read them only; the scale of
+    // output channel n is the largest |weight| of the channel over 448, the largest e4m3 value. A warp per channel
+    // (a thread per channel walked its 144 weights one by one and made this the longest part of every bf16 call: 31
+    // of 53 us of a 64-configuration log psi).
+    if (!f8) return;
+    const int lane = threadIdx.x & 31;
+    for (int e = tid >> 5; e < (p.n_layers - 1) * C; e += nth >> 5) {
         const int l = 1 + e / C, n = e - (l - 1) * C;
         const double *wn = params + layer_offset(p, l) + (size_t)n * C * 9;   // [cin][dy][dx] of channel n
         double m = 0.0;
-        for (int k = 0; k < 9 * C; ++k) m = fmax(m, fabs(wn[k]));
+        for (int k = lane; k < 9 * C; k += 32) m = fmax(m, fabs(wn[k]));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
         const float sc = m > 0.0 ? (float)m / 448.f : 1.f;
         // row-form image [pair q][K half h][column block j = 1 - dx][C][16 input channels]: kernel row
         // dy = 2 q + h (dy = 3: zero), so one K = 32 operand holds two kernel rows; then the scales
         unsigned char *dst = packed + pl.f32_bytes + pl.w0bytes + 2 * (size_t)(p.n_layers - 1) * pl.wbytes +
                              (size_t)(l - 1) * pl.f8bytes;
-        reinterpret_cast<float *>(dst + 12 * C * C)[n] = 0.5f * sc;   // halved, as the epilogue uses it
-        for (int q = 0; q < 2; ++q)
-            for (int h = 0; h < 2; ++h)
-                for (int j = 0; j < 3; ++j) {
-                    const int dy = 2 * q + h, dxi = 2 - j;
-                    unsigned short *row = reinterpret_cast<unsigned short *>(dst + (((q * 2 + h) * 3 + j) * C + n) * 16);
-                    for (int k = 0; k < 16; k += 2) {
-                        const float w0 = dy < 3 ? (float)wn[k * 9 + dy * 3 + dxi] / sc : 0.f;
-                        const float w1 = dy < 3 ? (float)wn[(k + 1) * 9 + dy * 3 + dxi] / sc : 0.f;
-                        row[k / 2] = (unsigned short)ptx::pack_e4m3(w0, w1);
-                    }
-                }
+        if (lane == 0) reinterpret_cast<float *>(dst + 12 * C * C)[n] = 0.5f * sc;   // halved, as the epilogue uses it
+        for (int t = lane; t < 4 * 3 * 8; t += 32) {   // (kernel row, column block, pair of input channels)
+            const int dy = t / 24, j = t / 8 % 3, k = 2 * (t & 7), dxi = 2 - j;
+            unsigned short *row = reinterpret_cast<unsigned short *>(dst + ((dy * 3 + j) * C + n) * 16);
+            const float w0 = dy < 3 ? (float)wn[k * 9 + dy * 3 + dxi] / sc : 0.f;
+            const float w1 = dy < 3 ? (float)wn[(k + 1) * 9 + dy * 3 + dxi] / sc : 0.f;
+            row[k / 2] = (unsigned short)ptx::pack_e4m3(w0, w1);
+        }
     }
 }
 
@@ -2828,18 +2829,36 @@ size_t tc_packed_bytes(const Problem &p) {
     return pl.f32_bytes + pl.w0bytes + 2 * (size_t)(p.n_layers - 1) * pl.wbytes + (size_t)(p.n_layers - 1) * pl.f8bytes;
 }
 
-int launch_tc_pack(const Problem &p, const double *p64, void *packed, const LaunchEnv &env) {
+int launch_tc_pack(const Problem &p, const double *p64, void *packed, bool f8, const LaunchEnv &env) {
     std::string why;
     if (!tc_supported(p, &why)) { *env.msg = why; return NQS_ERR_UNSUPPORTED; }
     TcPlan pl{};
     plan_weights(p, pl);
-    tc_pack_kernel<<<64, 256, 0, env.stream>>>(p, pl, p64, (unsigned char *)packed);
+    // a thread per weight, up to two blocks per SM
+    const int blocks = std::max(1, std::min((p.P + 255) / 256, 2 * env.num_sms));
+    tc_pack_kernel<<<blocks, 256, 0, env.stream>>>(p, pl, p64, (unsigned char *)packed, f8 && pl.f8bytes > 0);
     return check(env, "tc_pack_kernel");
 }
 
 #define NQS_TC_DISPATCH(C, ...)                                      \
     if ((C) == 16) { constexpr int CC = 16; __VA_ARGS__; }            \
     else { constexpr int CC = 32; __VA_ARGS__; }
+
+// A call with at most half the configurations that the plan's groups would
+// hold takes the smallest group that still gives every configuration a block
+// at once: a group's layers are a chain of latencies that grows with its tiles
+// (a whole call of 64 configurations at 10x10, with the packing of the
+// parameters: 53.8 us in eight groups of eight, 17.2 us in 64 of one, of which
+// the packing gave about two thirds).
+void logpsi_group(const Problem &p, int64_t n, int num_sms, size_t max_smem, TcPlan *pl) {
+    int fg, fs, fc;
+    if (forced_plan(&fg, &fs, &fc)) return;
+    const int64_t blocks = (int64_t)num_sms * pl->ctas;
+    const int64_t G = std::max<int64_t>(1, (n + blocks - 1) / blocks);
+    TcPlan small;
+    std::string why;
+    if (2 * G <= pl->G * pl->slots && make_plan(p, (int)G, 1, pl->ctas, max_smem, 0, &small, &why)) *pl = small;
+}
 
 int launch_logpsi_tc(const Problem &p, const double *, const void *packed, const int8_t *configs, int64_t n,
                      double *out, const LaunchEnv &env) {
@@ -2850,6 +2869,7 @@ int launch_logpsi_tc(const Problem &p, const double *, const void *packed, const
         *env.msg = why;
         return NQS_ERR_UNSUPPORTED;
     }
+    logpsi_group(p, n, env.num_sms, env.max_smem, &pl);
     const int64_t per = pl.G * pl.slots;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, (int64_t)env.num_sms * pl.ctas));
     NQS_TC_DISPATCH(p.C, {
@@ -3155,6 +3175,7 @@ int tc_describe_plan(const Problem &p, int kind, int64_t n, size_t max_smem, int
         if (kind == 2) ok = sample_plan(p, max_smem, n, num_sms, &pl, &per_block, why);
         else if (kind == 1 && use_row_form(p, max_smem, false, &pl)) ok = true;
         else ok = best_plan(p, max_smem, kind == 1, 16, 2, &pl, why);
+        if (ok && kind == 0) logpsi_group(p, n, num_sms, max_smem, &pl);
     }
     if (!ok) return NQS_ERR_UNSUPPORTED;
     const int64_t per = (int64_t)pl.G * pl.slots, cap = (int64_t)num_sms * pl.ctas;
