@@ -1077,13 +1077,15 @@ __host__ __device__ inline size_t wide_cache_bytes(const TcPlan &pl) {
 // interior MMA, so that one thread issues as fast as the operand path takes
 // them (45 cycles at N = 48, 54 at N = 96 on an idle SM; 66 and 57 with the
 // columns in one loop; the election in every MMA cost 8 - 17 % of the whole
-// kernel). False if the wait for the weights gave up.
+// kernel). All of that is computed before the wait for the stage: it stood
+// between the stage and the first MMA, ~500 cycles a layer (11.02 -> 10.85 ms
+// for 8,192 samples at 10 x 10 x 16 channels, 67.8 -> 64.9 ms for 4,096 at
+// 16 x 16 x 32). False if a wait gave up.
 template <int C>
 __device__ bool wide_issue(const TcPlan &pl, const TcShared &sh, const unsigned char *packed, const TcState &st, int l,
-                           int iw, int cls) {
+                           int iw, int cls, uint32_t ready) {
     const uint32_t q = __shfl_sync(0xffffffffu, st.wseq + (uint32_t)l, 0);
     if (!__all_sync(0xffffffffu, wide_wait(&sh.bar_w[q & 1], (q >> 1) & 1, sh.abort_flag))) return false;
-    ptx::tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *sh.tmem_addr, 0);
     const uint32_t wb = ptx::smem_u32(sh.base + ((q & 1) ? pl.o_w1 : pl.o_w0));
     const uint32_t abase = desc_lo(row_act(pl, sh), pl.plane), kplane = pl.plane >> 3;   // two planes, 16-byte units
@@ -1093,19 +1095,22 @@ __device__ bool wide_issue(const TcPlan &pl, const TcShared &sh, const unsigned 
     int lo, hi;
     wide_cols(pl, cls, l, lo, hi);
     const int L = pl.L, H = L / 2, xa = iw == 0 ? lo : H, xb = iw == 0 ? H : hi + 1;
+    const uint32_t step = (uint32_t)(pl.Lp * pl.G), bbase = desc_lo(wb, (l == 0 ? 1 : 3) * C * 16);
+    const uint32_t left = (uint32_t)(xa == 0 ? L - 1 : xa - 1) * step, right = (uint32_t)(xb == L ? 0 : xb) * step;
+    const uint32_t dl = tmem + (uint32_t)(xa * C), dr = tmem + (uint32_t)((xb - 1) * C);
+    const uint64_t z = dh | desc_lo(ptx::smem_u32(sh.base + pl.o_zero), 2048);
+    const uint32_t izero = ptx::idesc_bf16(128, (xb - xa) * C);
+    // stage 1 (A) or 2 (B) of the layer before: this half's input is written, its accumulators are drained
+    if (l > 0 && !__all_sync(0xffffffffu, wide_wait(&sh.bar_tile[2 + iw], ready, sh.abort_flag))) return false;
+    ptx::tc_fence_after();
     if (ptx::elect_one()) {
         if (l == 0) {
-            const uint32_t bbase = desc_lo(wb, C * 16);
             uint32_t a = abase + (uint32_t)(xa * 128), d = tmem + (uint32_t)(xa * C);
             for (int x = xa; x < xb; ++x, a += 128u, d += C)
                 for (int kk = 0; kk < pl.K0 / 16; ++kk)
                     ptx::mma_bf16(d, dh | (a + kk * kplane), dh | (bbase + (uint32_t)(2 * kk * C)), i1, kk ? 1u : 0u);
         } else {
-            const uint64_t z = dh | desc_lo(ptx::smem_u32(sh.base + pl.o_zero), 2048);
-            ptx::mma_bf16(tmem + (uint32_t)(xa * C), z, z, ptx::idesc_bf16(128, (xb - xa) * C), 0u);
-            const uint32_t bbase = desc_lo(wb, 3 * C * 16), step = (uint32_t)(pl.Lp * pl.G);
-            const uint32_t left = (uint32_t)(xa == 0 ? L - 1 : xa - 1) * step, right = (uint32_t)(xb == L ? 0 : xb) * step;
-            const uint32_t dl = tmem + (uint32_t)(xa * C), dr = tmem + (uint32_t)((xb - 1) * C);
+            ptx::mma_bf16(dl, z, z, izero, 0u);
             auto one = [&](uint32_t a, uint32_t b, uint32_t d, uint32_t idesc) {
 #pragma unroll
                 for (int kk = 0; kk < C / 16; ++kk)
@@ -1164,18 +1169,35 @@ struct WideCfg {
     int16_t i, j, roll, pad;
 };
 
+// The group's configurations: entries first .. first + count - 1 of the
+// connected list in evaluation order (negative: the sample itself; slots past
+// count repeat it). cfgs holds them for groups with a class (their rolls).
+struct WideEntries {
+    const int16_t *ci, *cj, *ord;
+    const WideCfg *cfgs;
+    int first, count, cls;
+    __device__ __forceinline__ WideCfg get(int g) const {
+        if (cls >= 0) return cfgs[g];
+        if (g >= count || first + g < 0) return WideCfg{-1, -1, 0, 0};
+        const int k = ord[first + g];
+        return WideCfg{ci[k], cj[k], 0, 0};
+    }
+    __device__ __forceinline__ int roll(int g) const { return cls < 0 ? 0 : cfgs[g].roll; }
+};
+
 // Layer-0 im2col of columns lo .. hi: row x * 128 + m (m = y * G + g), K0
 // columns tap-major (one-hot channel minor), straight from the sample with
 // each row's exchange and roll applied. A group of 128 threads walks its share
-// of the columns with the 3 x 3 window in registers (three loads a column).
-__device__ void wide_build(const TcPlan &pl, const TcShared &sh, const int8_t *sigma, const WideCfg *cfgs, int lo,
+// of the columns with the 3 x 3 window in registers (three loads a column, the
+// next column's ahead of the current one's stores).
+__device__ void wide_build(const TcPlan &pl, const TcShared &sh, const int8_t *sigma, const WideEntries &ent, int lo,
                            int hi) {
     const int L = pl.L, groups = (int)(blockDim.x >> 7), grp = (int)(threadIdx.x >> 7), n = hi - lo + 1;
     const int xb = lo + grp * n / groups, xe = grp < groups ? lo + (grp + 1) * n / groups : xb;
     const int m = threadIdx.x & 127;
     const WideRow w = wide_row(pl, sh, m);
     if (xb < xe && w.valid) {
-        const WideCfg cf = cfgs[w.g];
+        const WideCfg cf = ent.get(w.g);
         const int i = cf.i, j = cf.j;
         const int r0 = (w.y == 0 ? L - 1 : w.y - 1) * L, r1 = w.y * L, r2 = (w.y == L - 1 ? 0 : w.y + 1) * L;
         auto at = [&](int site) -> uint32_t {   // the site's value after the exchange, as an unsigned byte
@@ -1434,58 +1456,58 @@ __device__ bool wide_epilogue(const TcPlan &pl, const TcShared &sh, const WideRo
 
 // Sums of the head contributions per configuration, in head_slot's order
 // (lane k takes the original sites k, k + 32, ..., then the xor-shuffle tree);
-// one warp per configuration and output.
-__device__ void wide_head(const TcPlan &pl, const TcShared &sh, const WideCfg *cfgs) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = pl.G, L = pl.L;
+// one warp per configuration and output, the sites' addresses from the table of
+// row_bind (offset of the canonical site, its column in the top bits) instead
+// of two divisions' worth of steps a site: with the lists read in place below,
+// 6.46 -> 6.23 ms for five 8- to 16-site lattices in one launch, 64.9 -> 64.6 ms
+// at 16 x 16 x 32 channels, 10.9 ms either way at 10 x 10 x 16. (Both outputs
+// in one warp: 7.14 -> 7.02 ms at 12 x 12, but 10.9 -> 11.3 ms at 10 x 10.)
+__device__ void wide_head(const TcPlan &pl, const TcShared &sh, const WideEntries &ent) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = pl.G, L = pl.L, N = pl.N;
     const float *contrib = reinterpret_cast<const float *>(sh.base + pl.o_act);
-    const int y0 = lane / L, x0 = lane - y0 * L, dy = 32 / L, dx = 32 - dy * L, colw = pl.Lp * G * 4 + 1;
-    for (int t = warp; t < 2 * G; t += (int)(blockDim.x >> 5)) {
-        const int g = t >> 1;
-        const float *src = contrib + (t & 1) * L * G + g;
-        int c = x0 - cfgs[g].roll, y = y0;   // canonical column, row of the lane's site
-        if (c < 0) c += L;
-        int x = x0;
-        float sum = 0.f;
-        for (int site = lane; site < pl.N; site += 32) {
-            sum += src[c * colw + y * G];
-            x += dx, y += dy, c += dx;
-            if (c >= L) c -= L;
-            if (x >= L) { x -= L; ++y; }
+    const uint32_t *tab = reinterpret_cast<const uint32_t *>(sh.base + pl.o_sitetab);
+    for (int gk = warp; gk < 2 * G; gk += (int)(blockDim.x >> 5)) {
+        const int g = gk >> 1, k = gk & 1;
+        const int r = ent.roll(g);
+        const float *src = contrib + k * L * G + g;
+        float s = 0.f;
+#pragma unroll 4
+        for (int site = lane; site < N; site += 32) {
+            uint32_t e = tab[site];
+            if (r) e = tab[site - r + ((int)(e >> 24) < r ? L : 0)];   // the column it was evaluated at
+            s += src[e & 0xFFFFFFu];
         }
 #pragma unroll
-        for (int k = 16; k > 0; k >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, k);
-        if (lane == 0) sh.res[(t & 1) * G + g] = (double)sum;
+        for (int m = 16; m > 0; m >>= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+        if (lane == 0) sh.res[k * G + g] = (double)s;
     }
     __syncthreads();
 }
 
-// Evaluate the group's G configurations (cfgs, of the sample sigma) in the
+// Evaluate the group's G configurations (entries of the sample sigma) in the
 // wide row form; results in sh.res. False if a wait gave up (the block must
 // stop).
 template <int C>
 __device__ bool wide_forward(const TcPlan &pl, const TcShared &sh, const unsigned char *packed, TcState &st, int *err,
-                             const int8_t *sigma, const WideCfg *cfgs, int cls, const unsigned char *cache,
+                             const int8_t *sigma, const WideEntries &ent, const unsigned char *cache,
                              unsigned char *cache_w) {
+    const int cls = ent.cls;
     {
         int lo, hi;
         wide_cols(pl, cls, 0, lo, hi);
-        wide_build(pl, sh, sigma, cfgs, lo, hi);
+        wide_build(pl, sh, sigma, ent, lo, hi);
     }
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), nl = pl.n_layers;
     uint32_t ph = st.tphase;
     bool ok = true;
     if (warp >= pl.epi + kIssuers) {
         for (int l = 0; ok && l < nl; ++l)
-            ok = wide_fill_layer<C>(pl, sh, ph, l, cls, cfgs, cache, warp - pl.epi - kIssuers);
+            ok = wide_fill_layer<C>(pl, sh, ph, l, cls, ent.cfgs, cache, warp - pl.epi - kIssuers);
     } else if (warp >= pl.epi) {
         const int iw = warp - pl.epi;
         for (int l = 0; ok && l < nl; ++l) {
-            if (l > 0) {   // stage 1 (A) or 2 (B) of the layer before: this half's input is written, its accumulators drained
-                ok = __all_sync(0xffffffffu,
-                                wide_wait(&sh.bar_tile[2 + iw], (ph >> (2 + iw)) & 1u, sh.abort_flag));
-                ph ^= 4u << iw;
-            }
-            ok = ok && wide_issue<C>(pl, sh, packed, st, l, iw, cls);
+            ok = wide_issue<C>(pl, sh, packed, st, l, iw, cls, (ph >> (2 + iw)) & 1u);
+            if (l > 0) ph ^= 4u << iw;
         }
     } else {
         const WideRow w = wide_row(pl, sh, threadIdx.x & 127);
@@ -1499,7 +1521,7 @@ __device__ bool wide_forward(const TcPlan &pl, const TcShared &sh, const unsigne
     __syncthreads();
     ptx::tc_fence_after();
     if (*(volatile int *)sh.abort_flag) return false;
-    wide_head(pl, sh, cfgs);
+    wide_head(pl, sh, ent);
     st.wseq += (uint32_t)nl;
     return true;
 }
@@ -1582,26 +1604,22 @@ __device__ bool wide_sample(const TcPlan &pl, const Problem &p, const TcShared &
                 const int k = e.ord[e0 + cnt - 1 - lead];
                 cls = e.ci[k] % L != e.cj[k] % L;
             }
-            if (threadIdx.x < G) {
-                const int c = threadIdx.x, q = e0 + c - lead;   // list position (-1: sigma)
-                WideCfg v{-1, -1, 0, 0};
-                if (c < cnt && q >= 0) {
-                    const int k = e.ord[q];
-                    if (NQS_INDEX_OK(k >= 0 && k < nconn && e.ci[k] >= 0 && e.ci[k] < N && e.cj[k] >= 0 && e.cj[k] < N,
-                                     err)) {
+            if (cls >= 0) {
+                if (threadIdx.x < G) {
+                    WideCfg v{-1, -1, 0, 0};
+                    if ((int)threadIdx.x < cnt) {
+                        const int k = e.ord[e0 + threadIdx.x - lead];
                         v.i = e.ci[k];
                         v.j = e.cj[k];
-                        if (cls >= 0) {   // the bond's first site is the left one: to column H - 1
-                            const int r = v.i % L - (L / 2 - 1);
-                            v.roll = (int16_t)(r < 0 ? r + L : r);
-                        }
+                        const int r = v.i % L - (L / 2 - 1);   // the bond's first site is the left one: to column H - 1
+                        v.roll = (int16_t)(r < 0 ? r + L : r);
                     }
+                    e.cfgs[threadIdx.x] = v;
                 }
-                e.cfgs[c] = v;
+                __syncthreads();
             }
-            __syncthreads();
-            if (!wide_forward<C>(pl, sh, packed, st, err, e.sigma, e.cfgs, cls, cache,
-                                 cone && lead && e0 == 0 ? cache : nullptr))
+            const WideEntries ent{e.ci, e.cj, e.ord, e.cfgs, e0 - lead, cnt, cls};
+            if (!wide_forward<C>(pl, sh, packed, st, err, e.sigma, ent, cache, cone && lead && e0 == 0 ? cache : nullptr))
                 return false;
             if (threadIdx.x < cnt) {
                 const int q = e0 + (int)threadIdx.x - lead, idx = q < 0 ? 0 : e.ord[q] + lead;
@@ -1718,7 +1736,13 @@ __device__ void row_bind(const TcPlan &pl, TcShared &sh, const unsigned char *pa
     // the wide form's epilogue reads halved biases
     const uint32_t halved = pl.rows == 2 ? (uint32_t)(pl.n_layers * pl.C) : 0u;
     for (uint32_t i = threadIdx.x; i < pl.f32_count; i += blockDim.x) sh.f32[i] = i < halved ? 0.5f * src[i] : src[i];
-    if (pl.rows == 2)
+    if (pl.rows == 2) {
+        // where the head contributions of site (x, y) lie (wide_contrib), and x
+        for (int site = threadIdx.x; site < pl.N; site += blockDim.x) {
+            const int y = site / pl.L, x = site - y * pl.L;
+            reinterpret_cast<uint32_t *>(smem + pl.o_sitetab)[site] =
+                (uint32_t)(wide_contrib(pl, x) + y * pl.G) | (uint32_t)x << 24;
+        }
         for (int m = threadIdx.x; m < 128; m += blockDim.x) {
             const bool valid = m < pl.G * pl.L;
             const int y = valid ? m / pl.G : 0, g = valid ? m - y * pl.G : 0;
@@ -1727,6 +1751,7 @@ __device__ void row_bind(const TcPlan &pl, TcShared &sh, const unsigned char *pa
                 make_int4(y | (g << 8) | ((int)valid << 16), ((y + 1) * pl.G + g) * 16,
                           yimg < 0 ? 0 : (yimg - (y + 1)) * pl.G * 16, 0);
         }
+    }
     // zero the activations (rows no output writes are read only by discarded
     // accumulator rows, but stay finite) and the zero block
     for (uint32_t i = threadIdx.x; i < pl.act_bytes / 4; i += blockDim.x)
@@ -2642,6 +2667,7 @@ bool make_wide_plan(const Problem &p, size_t max_smem, TcPlan *out, std::string 
     pl.o_w1 = o; o = al16(o + pl.wbytes);
     pl.o_f32 = o; o = al16(o + pl.f32_count * 4);
     pl.o_lane = o; o = al16(o + 16 * 128);
+    pl.o_sitetab = o; o = al16(o + 4 * p.N);
     pl.o_res = o; o = al16(o + 16 * pl.G);
     uint32_t extra;
     wide_extra(nullptr, p.N, bond_chunk(p), &extra);
