@@ -629,7 +629,7 @@ def eloc_algorithmic_flops(w, n_samples, pairs, n_conn):
 TRAFFIC_SOURCES = ('tc.cu', 'tc_ptx.cuh', 'common.cuh', 'internal.h')
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one E_loc launch captured by ncu under
 # `bench.py --profile-eloc 2048`, with the hash of the kernel sources it was taken on
-TRAFFIC_RECORD = {'kernel': 'eloc_rows_kernel', 'samples': 2048, 'dram_bytes': 741632,
+TRAFFIC_RECORD = {'kernel': 'eloc_wide_kernel', 'samples': 2048, 'dram_bytes': 741632,
                   'source_sha256': '0fd012c4aa373536d53f1a8048253b0b3e102dd888ca0e442bd0a904243f6ae1'}
 
 
@@ -983,7 +983,7 @@ def main():
         eloc_launch_s = float(eloc_ms.mean()) / 1000.0
         achieved = flops / eloc_launch_s / 1e12
         if args.precision == 'bf16':
-            eloc_kernel = ('eloc_rows_kernel' if nqs.tc_plan(prob, 'local_energy', n_samples)['row_form']
+            eloc_kernel = ('eloc_wide_kernel' if nqs.tc_plan(prob, 'local_energy', n_samples)['row_form']
                            else 'eloc_tc_kernel')
             peak = peaks.get('bf16_tflops_sustained') or peaks['bf16_tflops']
             roof = {'bound': 'tensor', 'achieved': achieved, 'peak': peak, 'unit': 'TFLOP/s',
@@ -1006,7 +1006,8 @@ def main():
             lanes = 128 if args.precision == 'fp32' else 2
             peak = 152 * lanes * 2 * mhz * 1e6 / 1e12
             roof = {'bound': 'alu', 'achieved': achieved, 'peak': peak, 'unit': 'TFLOP/s', 'frac': achieved / peak,
-                    'traffic': None, 'kernel': 'eloc_plain_kernel',
+                    'traffic': None,
+                    'kernel': 'eloc_f32_kernel' if args.precision == 'fp32' and w['channels'] >= 8 else 'eloc_plain_kernel',
                     'peak_source': '152 SMs x %d lanes x 2 FLOP x %.0f MHz' % (lanes, mhz),
                     'flops': 'cone form (changed sites only) %.4g per launch' % flops,
                     'dense_form': {'achieved': flops_dense / eloc_launch_s / 1e12,

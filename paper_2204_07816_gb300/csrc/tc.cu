@@ -12,7 +12,10 @@
 // one tcgen05.mma whose A descriptor starts at a shifted address (an
 // implicit GEMM with no im2col copy): M = 128 rows, N = C, K = 16.
 // Layer 0 (one spin channel, or three one-hot channels) instead reads a
-// small im2col matrix of the spins (K = 16 or 32).
+// small im2col matrix of the spins (K = 16 or 32). This is the tap form, used
+// by log psi, the sampler and the local energies that the other two do not
+// take; the row form and the wide row form of the local energies (their own
+// comments below) put the x positions along the accumulator's columns.
 //
 // Pipeline. Halo rows are refreshed by the epilogue, which writes every
 // interior output also to its periodic images (a per-row destination table
@@ -1038,9 +1041,10 @@ __device__ bool row_forward(const TcPlan &pl, const TcShared &sh, const unsigned
 // the N = 3C MMAs (128 x 96 x 16: 7 KB, 56 cycles, against 120 for the tap
 // form's three N = 32 MMAs), the epilogue's stores, which share it, and the
 // latency of the stages. Measured (GB300): J1-J2 16x16, 32 channels, 8 layers,
-// 4,096 samples 127.2 ms in the tap form, 75.2 dense and 67.9 with cones here;
-// t-J 12x12, 32 channels, 6 layers, 2,048 samples 10.97 -> 7.41; J1-J2 10x10,
-// 16 channels, 6 layers, 8,192 samples 12.27 in the row form -> 11.04.
+// 4,096 samples 127.2 ms in the tap form, 64.4 here (cones; 75.2 dense against
+// 67.9 with cones when those were added); t-J 12x12, 32 channels, 6 layers,
+// 2,048 samples 10.97 -> 7.04; J1-J2 10x10, 16 channels, 6 layers, 8,192
+// samples 12.27 in the row form -> 10.84.
 constexpr int kWideEpi = 16;    // epilogue warps with one block per SM (two blocks: kMaxEpiWarps each)
 // warps that copy the columns outside a band while the epilogue warps work (launches with cones only; they fit beside
 // the issuers in the register allocation's granule of four warps)
@@ -1188,8 +1192,7 @@ struct WideEntries {
 // Layer-0 im2col of columns lo .. hi: row x * 128 + m (m = y * G + g), K0
 // columns tap-major (one-hot channel minor), straight from the sample with
 // each row's exchange and roll applied. A group of 128 threads walks its share
-// of the columns with the 3 x 3 window in registers (three loads a column, the
-// next column's ahead of the current one's stores).
+// of the columns with the 3 x 3 window in registers (three loads a column).
 __device__ void wide_build(const TcPlan &pl, const TcShared &sh, const int8_t *sigma, const WideEntries &ent, int lo,
                            int hi) {
     const int L = pl.L, groups = (int)(blockDim.x >> 7), grp = (int)(threadIdx.x >> 7), n = hi - lo + 1;
@@ -1459,7 +1462,7 @@ __device__ bool wide_epilogue(const TcPlan &pl, const TcShared &sh, const WideRo
 // one warp per configuration and output, the sites' addresses from the table of
 // row_bind (offset of the canonical site, its column in the top bits) instead
 // of two divisions' worth of steps a site: with the lists read in place below,
-// 6.46 -> 6.23 ms for five 8- to 16-site lattices in one launch, 64.9 -> 64.6 ms
+// 6.46 -> 6.23 ms for six requests of 6 x 6 to 12 x 12 in one launch, 64.9 -> 64.6 ms
 // at 16 x 16 x 32 channels, 10.9 ms either way at 10 x 10 x 16. (Both outputs
 // in one warp: 7.14 -> 7.02 ms at 12 x 12, but 10.9 -> 11.3 ms at 10 x 10.)
 __device__ void wide_head(const TcPlan &pl, const TcShared &sh, const WideEntries &ent) {
@@ -3004,7 +3007,7 @@ size_t tc_multi_table_bytes(int count) { return 256 + sizeof(TcRequest) * (size_
 // plan in launches of up to kWideGroupMax problems, the others in one tap-form
 // launch. A mix of six requests (J1-J2 6x6 .. 12x12, t-J 6x6 and 12x12, both
 // channel counts, 4 layers, 512 - 2,048 samples): 11.8 ms with every problem in
-// the tap form at one block per SM, 6.6 ms this way.
+// the tap form at one block per SM, 6.2 ms this way.
 int launch_eloc_tc_multi(const TcMultiItem *items, int count, void *dev_table, int max_blocks, const LaunchEnv &env) {
     if (count <= 0) return NQS_OK;
     const int C = items[0].p.C;

@@ -40,6 +40,23 @@ def test_grouped_equals_single_problem_launches(prec):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize('count', [22, 24, 33])
+def test_grouped_many_requests(count):
+    """More requests than one launch of the wide form holds, with members of
+    the tap form between them: bitwise the single-problem launches."""
+    nqs = lib()
+    w = WL['j1j2_10x10']
+    kinds = [{'L': 6, 'n_up': 18, 'n_down': 18, 'channels': 32, 'n_layers': 2},
+             {'L': 8, 'n_up': 32, 'n_down': 32, 'channels': 32, 'n_layers': 2},
+             {'L': 4, 'n_up': 8, 'n_down': 8, 'channels': 32, 'n_layers': 2}]
+    ctxs = [make_ctx(w, param_seed=50 + i, **kinds[i % 7 % 3])[0] for i in range(count)]
+    cfgs = [dev(configs_for(w, 1 + i % 4, seed=60 + i, **kinds[i % 7 % 3])) for i in range(count)]
+    outs = nqs.local_energy_multi(ctxs, cfgs, 'bf16')
+    torch.cuda.synchronize()
+    for ctx, cfg, got in zip(ctxs, cfgs, outs):
+        assert torch.equal(got, ctx.local_energy(cfg, None, 'bf16'))
+
+
 def test_grouped_rejects_unsupported_channel_count():
     nqs = lib()
     w = WL['j1j2_4x4']

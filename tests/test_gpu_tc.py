@@ -64,6 +64,16 @@ def test_logpsi_bf16_independent_of_batch_slot(case):
     assert torch.equal(a1[:7], a3)
 
 
+@pytest.mark.parametrize('n', [1, 2, 151, 153, 305, 609])
+def test_logpsi_bf16_small_calls_equal_large(n):
+    """Calls that spread smaller groups over the SMs give bitwise the log psi
+    of a call that fills the groups."""
+    w = WL['j1j2_10x10']
+    ctx, _ = make_ctx(w)
+    x = dev(configs_for(w, 4096, seed=28))
+    assert torch.equal(ctx.logpsi(x[:n].contiguous(), 'bf16'), ctx.logpsi(x, 'bf16')[:n])
+
+
 @pytest.mark.parametrize('case', TC_CASES[:3], ids=_ids)
 def test_local_energy_bf16_energy_per_site(case):
     name, over = case
