@@ -1559,13 +1559,25 @@ __host__ __device__ inline WideExtra wide_extra(unsigned char *ex, int N, int ch
     return e;
 }
 
+// Set in block 0 of a cluster if a block gave up (a cluster has no cones, so
+// cfgs is free).
+__device__ __forceinline__ int *wide_gave_up(const WideExtra &e) { return reinterpret_cast<int *>(e.cfgs); }
+
+__device__ void tc_fini(TcShared &sh, TcState &st, uint32_t tmem_cols);
+
 // Local energy of one configuration through the wide row form: as eloc_sample
 // (the same terms in the same fixed order), with the group's configurations
-// described by their exchange and roll instead of copied.
+// described by their exchange and roll instead of copied. split blocks of a
+// cluster (no cones, a list of one chunk) take the groups in turn: each
+// enumerates the list and stores its entries' log psi into block 0's list; block
+// 0 sums. Each gives its tensor memory back before it waits for the others, so
+// that no block that holds some ever waits for one that may be waiting for some,
+// and meets the cluster's barrier also after a wait that gave up, so that block
+// 0 stays while others may write into it.
 template <int C>
-__device__ bool wide_sample(const TcPlan &pl, const Problem &p, const TcShared &sh, TcState &st,
+__device__ bool wide_sample(const TcPlan &pl, const Problem &p, TcShared &sh, TcState &st,
                             const unsigned char *packed, const int8_t *cfg, const double *logpsi_s, double *out_s,
-                            int *err, unsigned char *cache) {
+                            int *err, unsigned char *cache, int split = 1, int rank = 0) {
     const int G = pl.G, N = pl.N, L = pl.L, chunk = bond_chunk(p);
     uint32_t bytes;
     const WideExtra e = wide_extra(sh.base + pl.o_extra, N, chunk, &bytes);
@@ -1577,6 +1589,7 @@ __device__ bool wide_sample(const TcPlan &pl, const Problem &p, const TcShared &
     if (p.model == NQS_MODEL_TJ) snake_prefix(p, e.sigma, e.cum, *e.scr);
     double ref_a = 0.0, ref_phi = 0.0, hd_tot = 0.0, sr_tot = 0.0, si_tot = 0.0;   // identical in every thread
     if (!recompute) { ref_a = logpsi_s[0]; ref_phi = logpsi_s[1]; }
+    bool ok = true;
     for (int b0 = 0; b0 < p.n_bonds; b0 += chunk) {
         double hd;
         const int nconn = enumerate_range(p, e.sigma, b0, min(p.n_bonds, b0 + chunk), e.ci, e.cj, e.ch, &hd, e.cum,
@@ -1599,7 +1612,7 @@ __device__ bool wide_sample(const TcPlan &pl, const Problem &p, const TcShared &
                 base += tot;
             }
         __syncthreads();
-        for (int e0 = 0; e0 < n_entries; e0 += G) {
+        for (int e0 = rank * G; ok && e0 < n_entries; e0 += split * G) {
             const int cnt = min(G, n_entries - e0);
             // the group's class is its last entry's (class 1's band covers class 0); dense if it holds the sample
             int cls = -1;
@@ -1622,15 +1635,28 @@ __device__ bool wide_sample(const TcPlan &pl, const Problem &p, const TcShared &
                 __syncthreads();
             }
             const WideEntries ent{e.ci, e.cj, e.ord, e.cfgs, e0 - lead, cnt, cls};
-            if (!wide_forward<C>(pl, sh, packed, st, err, e.sigma, ent, cache, cone && lead && e0 == 0 ? cache : nullptr))
-                return false;
-            if (threadIdx.x < cnt) {
+            ok = wide_forward<C>(pl, sh, packed, st, err, e.sigma, ent, cache, cone && lead && e0 == 0 ? cache : nullptr);
+            if (ok && threadIdx.x < cnt) {
                 const int q = e0 + (int)threadIdx.x - lead, idx = q < 0 ? 0 : e.ord[q] + lead;
-                e.lp[2 * idx] = (float)sh.res[threadIdx.x];
-                e.lp[2 * idx + 1] = (float)sh.res[G + threadIdx.x];
+                const float la = (float)sh.res[threadIdx.x], lphi = (float)sh.res[G + threadIdx.x];
+                if (rank != 0) {
+                    ptx::st_cluster_v2f32(ptx::smem_u32(e.lp + 2 * idx), 0, la, lphi);
+                } else {
+                    e.lp[2 * idx] = la;
+                    e.lp[2 * idx + 1] = lphi;
+                }
             }
         }
-        __syncthreads();
+        if (split > 1) {
+            tc_fini(sh, st, pl.tmem_cols);
+            int *gave_up = wide_gave_up(e);
+            if (!ok && threadIdx.x == 0) ptx::st_cluster_b32(ptx::smem_u32(gave_up), 0, 1);
+            ptx::cluster_sync();   // block 0's list is complete; nothing is written into it from here on
+            if (rank != 0 || !ok || *gave_up != 0) return false;
+        } else {
+            if (!ok) return false;
+            __syncthreads();
+        }
         if (lead) { ref_a = (double)e.lp[0]; ref_phi = (double)e.lp[1]; }
         // off-diagonal terms in an order independent of the block size
         const double2 tsum = fixed_order_sum2(nconn, [&](int k) {
@@ -2042,6 +2068,25 @@ __global__ void __launch_bounds__(kWideThreads<C>, kWideBlocks<C>)
                             err, my_cache))
             break;
     tc_teardown(pl, sh, st);
+}
+
+// The same for few samples: a cluster of split blocks per sample, without cones
+// (wide_split chooses; the launch has exactly one cluster a sample).
+template <int C>
+__global__ void __launch_bounds__(kWideThreads<C>, kWideBlocks<C>)
+    eloc_wide_split_kernel(TcPlan pl, Problem p, const unsigned char *packed, const int8_t *configs,
+                           const double *logpsi, double *out, int *err, int split) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    TcShared sh;
+    TcState st;
+    uint32_t bytes;
+    if (threadIdx.x == 0) *wide_gave_up(wide_extra(smem + pl.o_extra, p.N, bond_chunk(p), &bytes)) = 0;
+    ptx::cluster_sync();   // every block of the cluster runs: its shared memory may be written
+    tc_init(sh, smem, pl.tmem_cols, st, (blockDim.x >> 5) - kIssuers);
+    row_bind(pl, sh, packed, st);
+    const int64_t s = blockIdx.x / (unsigned)split;
+    wide_sample<C>(pl, p, sh, st, packed, configs + s * p.N, logpsi ? logpsi + 2 * s : nullptr, out + 2 * s, err,
+                   nullptr, split, (int)(blockIdx.x % (unsigned)split));
 }
 
 // One problem of a grouped local-energy launch.
@@ -2936,6 +2981,38 @@ size_t tc_eloc_cache_bytes(const Problem &p, size_t max_smem, int num_sms, int64
     return (size_t)grid * sigma_cache_bytes(pl);
 }
 
+// Blocks per sample of a wide launch without cones: a call of few samples
+// leaves SMs idle while each of its blocks works through its sample's groups,
+// so 2, 4 or 8 blocks share a sample where all clusters are resident at once
+// and each block still has a group (half the bonds are connected, about).
+// Measured (GB300, ms a call, one block / 2 / 4 / 8 a sample): 10x10, 16
+// channels, 6 layers 0.377 / 0.199 / 0.114 / 0.081 for 8 samples, 0.379 / 0.199
+// / 0.114 / - for 34, 0.378 / 0.200 / 0.136 for 64, 0.396 / 0.234 for 140; t-J
+// 12x12, 32 channels, 8 samples 0.565 / 0.292 / 0.163 / 0.110; 14x14, 32
+// channels, 8 layers, 8 samples 1.73 / 0.89 / 0.48 / 0.26; 6x6, 16 channels,
+// 4 layers, 8 samples 0.092 / 0.057 / 0.048 / 0.048. NQS_TC_SPLIT=K caps it (1:
+// off).
+template <typename K>
+int wide_split(K kernel, const Problem &p, const TcPlan &pl, int64_t n, int num_sms, cudaLaunchConfig_t *cfg) {
+    const char *e = getenv("NQS_TC_SPLIT");
+    const int most = p.n_bonds > bond_chunk(p) ? 1 : (e ? atoi(e) : 8);
+    cfg->attrs[0].id = cudaLaunchAttributeClusterDimension;
+    cfg->attrs[0].val.clusterDim.y = cfg->attrs[0].val.clusterDim.z = 1;
+    cfg->numAttrs = 1;
+    for (int s = 8; s > 1; s /= 2) {
+        if (s > most || n * s > (int64_t)num_sms * pl.ctas || 2 * s * pl.G > p.n_bonds + 2 * pl.G) continue;
+        cfg->gridDim = dim3((unsigned)(n * s));
+        cfg->attrs[0].val.clusterDim.x = (unsigned)s;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kernel, cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            continue;
+        }
+        if (clusters * (int64_t)pl.ctas >= n) return s;   // the query counts one block per SM
+    }
+    return 1;
+}
+
 int launch_eloc_tc(const Problem &p, const double *, const void *packed, const int8_t *configs,
                    const double *logpsi, int64_t n, double *out, void *cache, size_t cache_bytes,
                    const LaunchEnv &env, bool f8) {
@@ -2970,10 +3047,27 @@ int launch_eloc_tc(const Problem &p, const double *, const void *packed, const i
             unsigned char *c = (need > 0 && cache && cache_bytes >= need) ? (unsigned char *)cache : nullptr;
             const int threads = 32 * (pl.epi + kIssuers + (c ? kWideFill : 0));
             NQS_TC_DISPATCH(p.C, {
-                auto k = eloc_wide_kernel<CC>;
-                if (int rc = prep(k, pl, env)) return rc;
-                k<<<grid, threads, pl.total, env.stream>>>(pl, p, (const unsigned char *)packed, configs, logpsi,
-                                                                    n, out, env.err, c);
+                int split = 1;
+                if (!c && 2 * n <= (int64_t)env.num_sms * pl.ctas) {
+                    auto k = eloc_wide_split_kernel<CC>;
+                    if (int rc = prep(k, pl, env)) return rc;
+                    cudaLaunchAttribute attr{};
+                    cudaLaunchConfig_t cfg{};
+                    cfg.blockDim = dim3((unsigned)threads);
+                    cfg.dynamicSmemBytes = pl.total;
+                    cfg.stream = env.stream;
+                    cfg.attrs = &attr;
+                    split = wide_split(k, p, pl, n, env.num_sms, &cfg);
+                    if (split > 1)
+                        (void)cudaLaunchKernelEx(&cfg, k, pl, p, (const unsigned char *)packed, configs, logpsi, out,
+                                                 env.err, split);   // check() below reports its error
+                }
+                if (split == 1) {
+                    auto k = eloc_wide_kernel<CC>;
+                    if (int rc = prep(k, pl, env)) return rc;
+                    k<<<grid, threads, pl.total, env.stream>>>(pl, p, (const unsigned char *)packed, configs, logpsi, n,
+                                                               out, env.err, c);
+                }
             });
             return check(env, "eloc_wide_kernel");
         }

@@ -348,6 +348,28 @@ __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.w
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Barrier of every thread of the cluster; shared-memory writes before it, also
+// into other blocks, are visible after it.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Store into the shared memory of block `rank` of the cluster, at this block's
+// address.
+__device__ __forceinline__ void st_cluster_v2f32(uint32_t addr, uint32_t rank, float a, float b) {
+    asm volatile(
+        "{\n\t.reg .b32 r;\n\t"
+        "mapa.shared::cluster.u32 r, %0, %1;\n\t"
+        "st.shared::cluster.v2.f32 [r], {%2, %3};\n\t}" ::"r"(addr), "r"(rank), "f"(a), "f"(b) : "memory");
+}
+
+__device__ __forceinline__ void st_cluster_b32(uint32_t addr, uint32_t rank, uint32_t v) {
+    asm volatile(
+        "{\n\t.reg .b32 r;\n\t"
+        "mapa.shared::cluster.u32 r, %0, %1;\n\t"
+        "st.shared::cluster.b32 [r], %2;\n\t}" ::"r"(addr), "r"(rank), "r"(v) : "memory");
+}
+
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }

@@ -208,6 +208,34 @@ def test_local_energy_wide_form_equals_tap_form(case, monkeypatch):
         assert torch.equal(got[key][0], got['tap'][0]) and torch.equal(got[key][1], got['tap'][1]), key
 
 
+SPLIT_CASES = [
+    ('j1j2_10x10', {}, 1), ('j1j2_10x10', {}, 19), ('j1j2_10x10', {}, 76), ('j1j2_10x10', {}, 152), ('j1j2_10x10', {}, 153),
+    ('j1j2_10x10', {'L': 9, 'n_up': 41, 'n_down': 40, 'n_layers': 3}, 37),
+    ('j1j2_16x16', {'n_layers': 2}, 5),
+    ('j1j2_16x16', {'L': 6, 'n_up': 18, 'n_down': 18, 'n_layers': 2}, 75),
+    ('tj_12x12', {}, 3), ('tj_12x12', {'n_layers': 2}, 38),
+]
+
+
+@pytest.mark.parametrize('case', SPLIT_CASES, ids=lambda c: '%s-%s-%d' % (c[0], '-'.join(map(str, c[1].values())), c[2]))
+def test_local_energy_few_samples_split_over_blocks(case, monkeypatch):
+    """Calls of few samples, each sample's connected list shared by the blocks of a cluster (two, four or eight, as
+    many as the rule takes at most): bitwise one block a sample, with log psi recomputed and supplied."""
+    name, over, n = case
+    w = WL[name]
+    ctx, _ = make_ctx(w, **over)
+    cfg = dev(configs_for(w, n, seed=45, **over))
+    lp = ctx.logpsi(cfg, 'bf16')
+    monkeypatch.setenv('NQS_TC_DENSE', '1')      # cones keep one block a sample
+    got = {}
+    for most in ('1', '2', '4', '8'):
+        monkeypatch.setenv('NQS_TC_SPLIT', most)
+        got[most] = ctx.local_energy(cfg, None, 'bf16'), ctx.local_energy(cfg, lp, 'bf16')
+    ctx.sync()
+    for most in ('2', '4', '8'):
+        assert torch.equal(got[most][0], got['1'][0]) and torch.equal(got[most][1], got['1'][1]), most
+
+
 def test_local_energy_bf16_zero_network():
     w = WL['j1j2_10x10']
     from tests.gpu_common import problem_of
