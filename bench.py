@@ -629,8 +629,8 @@ def eloc_algorithmic_flops(w, n_samples, pairs, n_conn):
 TRAFFIC_SOURCES = ('tc.cu', 'tc_ptx.cuh', 'common.cuh', 'internal.h')
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one E_loc launch captured by ncu under
 # `bench.py --profile-eloc 2048`, with the hash of the kernel sources it was taken on
-TRAFFIC_RECORD = {'kernel': 'eloc_wide_kernel', 'samples': 2048, 'dram_bytes': 741632,
-                  'source_sha256': '0fd012c4aa373536d53f1a8048253b0b3e102dd888ca0e442bd0a904243f6ae1'}
+TRAFFIC_RECORD = {'kernel': 'eloc_wide_kernel', 'samples': 2048, 'dram_bytes': 328960,
+                  'source_sha256': '7e54ebecccfe4415e413f9554e8b62c84197ae801393089b2ba324af9bf2d442'}
 
 
 def kernel_source_hash():
