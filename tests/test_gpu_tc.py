@@ -438,6 +438,36 @@ def test_sampler_ahead_equals_one_proposal_at_a_time(case, monkeypatch):
         assert n == n0 and c[1] == c0[1] and torch.equal(c[0], c0[0])
 
 
+@pytest.mark.parametrize('case', [('j1j2_10x10', {'channels': 32}, 64, 3.0), ('j1j2_10x10', {'L': 8, 'n_up': 32, 'n_down': 32, 'channels': 32}, 64, 2.0),
+                                  ('j1j2_10x10', {'L': 6, 'n_up': 18, 'n_down': 18}, 1024, 3.0)],
+                         ids=lambda c: '%d-%d' % (c[1].get('L', 10), c[2]))
+def test_sampler_ahead_pays_where_almost_every_move_is_rejected(case, monkeypatch):
+    """One sweep a call (as the server samples) on a strongly structured wave function: the prediction has to find
+    within a few forwards that moves are rejected, so that evaluating ahead is no slower than one proposal at a time
+    (0.7 to 0.9 of its time; 1.1 to 1.2 where the prediction starts each call far off and moves in small steps)."""
+    name, over, chains, scale = case
+    ctx, _ = make_ctx(WL[name], seed=3, scale=scale, **over)
+    ctx.sample(chains, 1, 1, 10, 'bf16')
+    ctx.sampler_counts(reset=True)
+    best = {}
+    for ahead in ('1', None) * 4:
+        if ahead:
+            monkeypatch.setenv('NQS_TC_AHEAD', ahead)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        ctx.sample(chains, 1, 1, 0, 'bf16')
+        a.record()
+        for _ in range(20):
+            ctx.sample(chains, 1, 1, 0, 'bf16')
+        b.record()
+        torch.cuda.synchronize()
+        best[ahead] = min(best.get(ahead, 1e9), a.elapsed_time(b))
+        if ahead:
+            monkeypatch.delenv('NQS_TC_AHEAD')
+    moves, accepted = ctx.sampler_counts()
+    assert accepted < 0.05 * moves
+    assert best[None] <= best['1']
+
+
 def nqs_param_count_of(w, **over):
     from tests.gpu_common import problem_of
     return lib().nqs_param_count(problem_of(w, **over))
