@@ -237,8 +237,10 @@ int nqs_local_energy(nqs_ctx *ctx, const int8_t *configs, const double *logpsi, 
  * Hamiltonians). Entry i evaluates what nqs_local_energy(ctxs[i],
  * configs[i], logpsi ? logpsi[i] : NULL, n[i], eloc_out[i], precision)
  * evaluates, with bitwise the same results. With NQS_BF16 the problems that
- * share a channel count run in one tensor-core launch whose blocks move from
- * problem to problem; the CUDA-core precisions run one launch per problem.
+ * share a channel count run in grouped tensor-core launches whose blocks move
+ * from problem to problem (one for each form of the network, a further one
+ * past 220 problems or 24 shapes of a form); the CUDA-core precisions run one
+ * launch per problem.
  * All work is enqueued on the stream of ctxs[0], which must be on the same
  * device as the others; the caller orders it after the work that produces
  * the inputs (e.g. with events). Host arrays of `count` entries; device

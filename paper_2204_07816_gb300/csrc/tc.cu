@@ -31,6 +31,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstring>
 #include <cstdlib>
 
 #include <vector>
@@ -2105,12 +2106,29 @@ struct TcRequest {
 // the single-problem kernel: descriptors stay in uniform registers). Blocks
 // take samples one at a time from a global counter in problem-major order and
 // re-bind their shared-memory plan when the problem changes. Dense: cones pay
-// only on the largest lattices.
-constexpr int kWideGroupMax = 16;
-struct WideGroup {
-    int count;
-    TcRequest r[kWideGroupMax];
+// only on the largest lattices. Requests of one shape share a plan, so that
+// the 32,764 bytes of a kernel's parameters hold more requests than there are
+// SMs: a launch of fewer would leave SMs idle that one launch of every request
+// keeps busy (32 channels, six layers, one to four samples a request, ms for 33
+// / 120 / 250 requests of 10x10 and 12x12: 2.19 / 7.17 / 14.7 in launches of 16,
+// 0.98 / 2.14 / 4.92 here, 1.71 / 3.68 / 7.51 in one tap-form launch).
+constexpr int kWideGroupPlans = 24;
+constexpr int kWideGroupMax = 220;
+struct WideRequest {
+    Problem p;
+    const unsigned char *packed;
+    const int8_t *configs;
+    const double *logpsi;
+    double *out;
+    int64_t start;   // index of the request's first sample in the launch
+    int plan;
 };
+struct WideGroup {
+    int count, plans;
+    TcPlan pl[kWideGroupPlans];
+    WideRequest r[kWideGroupMax];
+};
+static_assert(sizeof(WideGroup) + 64 <= 32764, "the requests are kernel parameters");
 
 template <int C>
 __global__ void __launch_bounds__(kWideThreads<C>, kWideBlocks<C>)
@@ -2128,16 +2146,21 @@ __global__ void __launch_bounds__(kWideThreads<C>, kWideBlocks<C>)
         const int64_t g = __shfl_sync(0xffffffffu, grab, 0);
         __syncthreads();
         if (g >= total) break;
-        int r = 0;
-        while (r + 1 < grp.count && grp.r[r + 1].start <= g) ++r;
-        const TcRequest &q = grp.r[r];
+        int r = max(cur, 0);   // a block's samples come in order
+        for (int end = grp.count; r + 1 < end;) {   // the last request that starts at or before sample g
+            const int mid = (r + end) / 2;
+            if (grp.r[mid].start <= g) r = mid;
+            else end = mid;
+        }
+        const WideRequest &q = grp.r[r];
+        const TcPlan &pl = grp.pl[__shfl_sync(0xffffffffu, q.plan, 0)];   // the index in a register, not read at every use
         if (r != cur) {
             if (cur >= 0) tc_unbind(sh, st);
-            row_bind(q.pl, sh, q.packed, st);
+            row_bind(pl, sh, q.packed, st);
             cur = r;
         }
         const int64_t s = g - q.start;
-        if (!wide_sample<C>(q.pl, q.p, sh, st, q.packed, q.configs + s * q.p.N, q.logpsi ? q.logpsi + 2 * s : nullptr,
+        if (!wide_sample<C>(pl, q.p, sh, st, q.packed, q.configs + s * q.p.N, q.logpsi ? q.logpsi + 2 * s : nullptr,
                             q.out + 2 * s, err, nullptr))
             break;
     }
@@ -3118,15 +3141,28 @@ size_t tc_multi_table_bytes(int count) { return 256 + sizeof(TcRequest) * (size_
 // plan in launches of up to kWideGroupMax problems, the others in one tap-form
 // launch. A mix of six requests (J1-J2 6x6 .. 12x12, t-J 6x6 and 12x12, both
 // channel counts, 4 layers, 512 - 2,048 samples): 11.8 ms with every problem in
-// the tap form at one block per SM, 6.2 ms this way.
+// the tap form at one block per SM, 6.2 ms this way. The launches follow each
+// other, so where all samples have an SM at once the longest tap-form sample
+// hides the others: then every problem takes the tap form if that is shorter
+// than the two launches by the samples' dense work (a wide sample takes 0.7 of
+// its tap-form time at 16 channels, 0.55 at 32: 10x10, six layers, 10 samples).
+// 10x10 and 16x16, 16 channels, six layers, 10 samples of four requests: 2.33
+// ms in two launches, 2.00 in one.
 int launch_eloc_tc_multi(const TcMultiItem *items, int count, void *dev_table, int max_blocks, const LaunchEnv &env) {
     if (count <= 0) return NQS_OK;
     const int C = items[0].p.C;
-    std::vector<TcRequest> tap, wide;
+    struct Member {
+        TcRequest r;   // with the tap form's plan
+        TcPlan wide;   // rows = 0: no wide plan
+    };
+    std::vector<Member> members;
+    int64_t samples = 0;
+    double longest[2] = {0.0, 0.0};   // dense work of a sample: tap form only, wide form
     for (int i = 0; i < count; ++i) {
         const Problem &p = items[i].p;
         std::string why;
-        TcRequest r;
+        Member m{};
+        TcRequest &r = m.r;
         if (p.C != C || !tc_supported(p, &why) || !best_plan(p, env.max_smem, true, 16, 1, &r.pl, &why)) {
             *env.msg = p.C != C ? std::string("grouped local energy needs one channel count per launch") : why;
             return NQS_ERR_UNSUPPORTED;
@@ -3138,10 +3174,20 @@ int launch_eloc_tc_multi(const TcMultiItem *items, int count, void *dev_table, i
         r.out = items[i].out;
         r.n = items[i].n;
         if (r.n == 0) continue;
-        TcPlan own;
-        const bool is_wide = use_row_form(p, env.max_smem, false, &own) && own.rows == 2;
-        if (is_wide) r.pl = own;
-        (is_wide ? wide : tap).push_back(r);
+        if (!use_row_form(p, env.max_smem, false, &m.wide) || m.wide.rows != 2) m.wide = TcPlan{};
+        double &most = longest[m.wide.rows == 2];
+        most = std::max(most, (double)p.n_bonds * p.N * p.n_layers);
+        samples += r.n;
+        members.push_back(m);
+    }
+    const int64_t slots = max_blocks > 0 ? std::min(max_blocks, env.num_sms) : env.num_sms;
+    const bool all_tap = longest[0] > 0.0 && samples <= slots &&
+                         std::max(longest[0], longest[1]) < longest[0] + (C == 16 ? 0.7 : 0.55) * longest[1];
+    std::vector<TcRequest> tap;
+    std::vector<const Member *> wide;
+    for (const Member &m : members) {
+        if (m.wide.rows == 2 && !all_tap) wide.push_back(&m);
+        else tap.push_back(m.r);
     }
     unsigned long long *counter = (unsigned long long *)dev_table;
     auto reset = [&]() -> int {
@@ -3154,20 +3200,23 @@ int launch_eloc_tc_multi(const TcMultiItem *items, int count, void *dev_table, i
         const int64_t most = (int64_t)env.num_sms * ctas;
         return (int)std::max<int64_t>(1, std::min(total, max_blocks > 0 ? std::min<int64_t>(max_blocks, most) : most));
     };
-    for (size_t w0 = 0; w0 < wide.size(); w0 += kWideGroupMax) {
+    for (size_t w0 = 0; w0 < wide.size();) {
         WideGroup grp{};
         uint32_t smem = 0, cols = 32;
         int64_t total = 0;
-        grp.count = (int)std::min<size_t>(kWideGroupMax, wide.size() - w0);
-        for (int i = 0; i < grp.count; ++i) {
-            TcRequest &r = grp.r[i] = wide[w0 + i];
-            r.start = total;
-            total += r.n;
-            smem = std::max(smem, r.pl.total);   // each plan already keeps to its blocks per SM
-            cols = std::max(cols, r.pl.tmem_cols);
+        for (; w0 < wide.size() && grp.count < kWideGroupMax; ++w0, ++grp.count) {
+            const Member &m = *wide[w0];
+            int k = 0;
+            while (k < grp.plans && std::memcmp(&grp.pl[k], &m.wide, sizeof(TcPlan)) != 0) ++k;
+            if (k == kWideGroupPlans) break;
+            if (k == grp.plans) grp.pl[grp.plans++] = m.wide;
+            grp.r[grp.count] = WideRequest{m.r.p, m.r.packed, m.r.configs, m.r.logpsi, m.r.out, total, k};
+            total += m.r.n;
+            smem = std::max(smem, m.wide.total);   // each plan already keeps to its blocks per SM
+            cols = std::max(cols, m.wide.tmem_cols);
         }
         if (int rc = reset()) return rc;
-        const int grid = grid_of(total, grp.r[0].pl.ctas), threads = 32 * (grp.r[0].pl.epi + kIssuers);
+        const int grid = grid_of(total, grp.pl[0].ctas), threads = 32 * (grp.pl[0].epi + kIssuers);
         NQS_TC_DISPATCH(C, {
             auto k = eloc_wide_multi_kernel<CC>;
             if (int rc = allow_dynamic_smem(k, smem, env)) return rc;

@@ -89,3 +89,43 @@ def test_chunked_enumeration_36x36_zero_network():
     ctx, _ = make_ctx(w, params=np.zeros(P), **over)
     e = ctx.local_energy(dev(configs_for(w, 3, seed=31, **over)), None, 'bf16').cpu().numpy()
     assert np.all(e[:, 0] == 0.75 * 1296) and np.all(e[:, 1] == 0.0)
+
+
+def _grouped(shapes, w='j1j2_10x10', cap=0):
+    """(contexts, configurations, grouped energies, launches of the grouped call) of requests (overrides, samples)."""
+    nqs = lib()
+    ctxs = [make_ctx(WL[w], param_seed=70 + i, **over)[0] for i, (over, _) in enumerate(shapes)]
+    cfgs = [dev(configs_for(WL[w], n, seed=80 + i, **over)) for i, (over, n) in enumerate(shapes)]
+    before = ctxs[0].kernel_launches()
+    outs = nqs.local_energy_multi(ctxs, cfgs, 'bf16', max_blocks=cap)
+    return ctxs, cfgs, outs, ctxs[0].kernel_launches() - before
+
+
+def _square(L, channels, layers):
+    return {'L': L, 'n_up': L * L // 2, 'n_down': L * L - L * L // 2, 'channels': channels, 'n_layers': layers}
+
+
+GROUPS = {
+    # one launch holds them all (beside one packing launch a request)
+    'many': ([(_square(6 + 2 * (i % 2), 32, 2), 1 + i % 4) for i in range(33)], 1),
+    'most': ([(_square(6, 16, 4), 1) for i in range(220)], 1),
+    'one more': ([(_square(6, 16, 4), 1) for i in range(221)], 2),
+    # more plans than a launch holds
+    'plans': ([(_square(L, 32, nl), 2) for nl in (1, 2, 3) for L in (6, 7, 8, 9, 10, 11, 12, 13, 14)], 2),
+    # few samples, some of them in the tap form only: everything in the tap form, if that is shorter
+    'beside longer': ([(_square(10, 16, 4), 3), (_square(16, 16, 4), 2)], 1),
+    'beside shorter': ([(_square(8, 32, 4), 3), (_square(4, 32, 4), 2)], 2),
+    'many samples': ([(_square(8, 16, 4), 160), (_square(16, 16, 2), 2)], 2),
+}
+
+
+@pytest.mark.parametrize('name', list(GROUPS))
+def test_grouped_launches(name):
+    """How many launches a grouped call takes (requests, plans and forms a launch holds), and bitwise the
+    single-problem launches, whichever form a request runs in."""
+    shapes, launches = GROUPS[name]
+    ctxs, cfgs, outs, count = _grouped(shapes)
+    torch.cuda.synchronize()
+    assert count == len(shapes) + launches
+    for ctx, cfg, got in zip(ctxs, cfgs, outs):
+        assert torch.equal(got, ctx.local_energy(cfg, None, 'bf16'))
