@@ -3196,10 +3196,9 @@ int launch_eloc_tc_multi(const TcMultiItem *items, int count, void *dev_table, i
         *env.msg = std::string("grouped counter: ") + cudaGetErrorString(e);
         return NQS_ERR_CUDA;
     };
-    const auto grid_of = [&](int64_t total, int ctas) {
-        const int64_t most = (int64_t)env.num_sms * ctas;
-        return (int)std::max<int64_t>(1, std::min(total, max_blocks > 0 ? std::min<int64_t>(max_blocks, most) : most));
-    };
+    // max_blocks is a share in SMs: the blocks that fill one SM count as one (16 channels, 1,536 samples of 10x10 to
+    // 6x6 capped at all 152 SMs: 1.64 ms with 152 half-SM blocks, 1.01 with 304)
+    const auto grid_of = [&](int64_t total, int ctas) { return (int)std::max<int64_t>(1, std::min(total, slots * ctas)); };
     for (size_t w0 = 0; w0 < wide.size();) {
         WideGroup grp{};
         uint32_t smem = 0, cols = 32;

@@ -129,3 +129,27 @@ def test_grouped_launches(name):
     assert count == len(shapes) + launches
     for ctx, cfg, got in zip(ctxs, cfgs, outs):
         assert torch.equal(got, ctx.local_energy(cfg, None, 'bf16'))
+
+
+def test_grouped_cap_is_a_share_of_the_sms():
+    """max_blocks counts SMs, also for the form whose blocks take half an SM each: capped at every SM a call is no
+    slower than uncapped (1.6 times where it gets half the blocks), and a cap changes no bit."""
+    nqs = lib()
+    shapes = [(_square(10, 16, 4), 512), (_square(8, 16, 4), 512), (_square(6, 16, 4), 512)]
+    ctxs, cfgs, outs, _ = _grouped(shapes)
+    for cap in (1, 31):
+        few = [c[:40].contiguous() for c in cfgs]
+        for a, b in zip(nqs.local_energy_multi(ctxs, few, 'bf16', max_blocks=cap), outs):
+            assert torch.equal(a, b[:40])
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    best = {}
+    for cap in (0, sms) * 4:
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        nqs.local_energy_multi(ctxs, cfgs, 'bf16', outs=outs, max_blocks=cap)
+        a.record()
+        for _ in range(5):
+            nqs.local_energy_multi(ctxs, cfgs, 'bf16', outs=outs, max_blocks=cap)
+        b.record()
+        torch.cuda.synchronize()
+        best[cap] = min(best.get(cap, 1e9), a.elapsed_time(b))
+    assert best[sms] <= 1.15 * best[0]
