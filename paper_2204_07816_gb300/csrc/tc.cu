@@ -3142,12 +3142,25 @@ size_t tc_multi_table_bytes(int count) { return 256 + sizeof(TcRequest) * (size_
 // launch. A mix of six requests (J1-J2 6x6 .. 12x12, t-J 6x6 and 12x12, both
 // channel counts, 4 layers, 512 - 2,048 samples): 11.8 ms with every problem in
 // the tap form at one block per SM, 6.2 ms this way. The launches follow each
-// other, so where all samples have an SM at once the longest tap-form sample
-// hides the others: then every problem takes the tap form if that is shorter
-// than the two launches by the samples' dense work (a wide sample takes 0.7 of
-// its tap-form time at 16 channels, 0.55 at 32: 10x10, six layers, 10 samples).
-// 10x10 and 16x16, 16 channels, six layers, 10 samples of four requests: 2.33
-// ms in two launches, 2.00 in one.
+// other, so with few samples each waits for its own longest ones: every problem
+// takes the tap form unless the two launches are shorter by GroupTime's estimate
+// (of 222 random groups of both forms, 2 to 30 requests of 1 to 150 samples:
+// 0.1 % above the faster choice on average; always two launches 18 % above,
+// always one 13 %; of 400 others none over 5 % slower than the tap form alone.
+// 10x10 and 16x16, 16 channels, six layers, 10 samples: 2.33 ms in two
+// launches, 2.00 in one).
+struct GroupTime {
+    double most = 0.0, sum = 0.0;
+    int64_t n = 0;
+    void add(double sample, int64_t count) {
+        most = std::max(most, sample);
+        sum += sample * (double)count;
+        n += count;
+    }
+    // one sample a slot: the longest; more: their share of the slots and part of the longest at the end
+    double over(int64_t slots) const { return n <= slots ? most : std::max(most, sum / (double)slots + 0.3 * most); }
+};
+
 int launch_eloc_tc_multi(const TcMultiItem *items, int count, void *dev_table, int max_blocks, const LaunchEnv &env) {
     if (count <= 0) return NQS_OK;
     const int C = items[0].p.C;
@@ -3156,8 +3169,7 @@ int launch_eloc_tc_multi(const TcMultiItem *items, int count, void *dev_table, i
         TcPlan wide;   // rows = 0: no wide plan
     };
     std::vector<Member> members;
-    int64_t samples = 0;
-    double longest[2] = {0.0, 0.0};   // dense work of a sample: tap form only, wide form
+    GroupTime all, rest, fast;   // every request in the tap form; those that have to; the others in the wide form
     for (int i = 0; i < count; ++i) {
         const Problem &p = items[i].p;
         std::string why;
@@ -3175,14 +3187,19 @@ int launch_eloc_tc_multi(const TcMultiItem *items, int count, void *dev_table, i
         r.n = items[i].n;
         if (r.n == 0) continue;
         if (!use_row_form(p, env.max_smem, false, &m.wide) || m.wide.rows != 2) m.wide = TcPlan{};
-        double &most = longest[m.wide.rows == 2];
-        most = std::max(most, (double)p.n_bonds * p.N * p.n_layers);
-        samples += r.n;
+        // a sample's time in the tap form (its work with two layers' worth beside), and in the wide form: 32 channels
+        // 0.9 of it at 6x6, 0.68 at 8x8, 0.5 at 13x13; 16 channels below
+        const double t = (double)p.n_bonds * p.N * (p.n_layers + 2);
+        all.add(t, r.n);
+        if (m.wide.rows != 2) rest.add(t, r.n);
+        else fast.add(C == 16 ? t : t * std::min(0.9, std::max(0.5, 5.4 / p.L)), r.n);
         members.push_back(m);
     }
     const int64_t slots = max_blocks > 0 ? std::min(max_blocks, env.num_sms) : env.num_sms;
-    const bool all_tap = longest[0] > 0.0 && samples <= slots &&
-                         std::max(longest[0], longest[1]) < longest[0] + (C == 16 ? 0.7 : 0.55) * longest[1];
+    // 16 channels: 0.9 of the tap form's time while a block has its SM to itself, 1.1 and two blocks an SM beyond
+    const double split = rest.over(slots) + (C == 32 ? fast.over(slots)
+                                                     : (fast.n <= slots ? 0.9 * fast.most : 1.1 * fast.over(2 * slots)));
+    const bool all_tap = rest.n > 0 && split > 0.95 * all.over(slots);
     std::vector<TcRequest> tap;
     std::vector<const Member *> wide;
     for (const Member &m : members) {

@@ -112,10 +112,11 @@ GROUPS = {
     'one more': ([(_square(6, 16, 4), 1) for i in range(221)], 2),
     # more plans than a launch holds
     'plans': ([(_square(L, 32, nl), 2) for nl in (1, 2, 3) for L in (6, 7, 8, 9, 10, 11, 12, 13, 14)], 2),
-    # few samples, some of them in the tap form only: everything in the tap form, if that is shorter
+    # some requests in the tap form only: everything in the tap form, if that is shorter than two launches
     'beside longer': ([(_square(10, 16, 4), 3), (_square(16, 16, 4), 2)], 1),
     'beside shorter': ([(_square(8, 32, 4), 3), (_square(4, 32, 4), 2)], 2),
-    'many samples': ([(_square(8, 16, 4), 160), (_square(16, 16, 2), 2)], 2),
+    'many samples': ([(_square(8, 16, 4), 6000), (_square(16, 16, 2), 2)], 2),
+    'more than SMs': ([(_square(10, 16, 4), 150), (_square(16, 16, 4), 20)], 1),
 }
 
 
