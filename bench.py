@@ -983,8 +983,8 @@ def main():
         eloc_launch_s = float(eloc_ms.mean()) / 1000.0
         achieved = flops / eloc_launch_s / 1e12
         if args.precision == 'bf16':
-            eloc_kernel = ('eloc_wide_kernel' if nqs.tc_plan(prob, 'local_energy', n_samples)['row_form']
-                           else 'eloc_tc_kernel')
+            eloc_kernel = {'tap': 'eloc_tc_kernel', 'row': 'eloc_rows_kernel',
+                           'wide': 'eloc_wide_kernel'}[nqs.tc_plan(prob, 'local_energy', n_samples)['form']]
             peak = peaks.get('bf16_tflops_sustained') or peaks['bf16_tflops']
             roof = {'bound': 'tensor', 'achieved': achieved, 'peak': peak, 'unit': 'TFLOP/s',
                     'frac': achieved / peak, 'traffic': recorded_traffic(n_samples, eloc_kernel),

@@ -131,13 +131,22 @@ int64_t nqs_param_count(const nqs_problem *p);
  * group, whose next proposals may be evaluated ahead), groups in flight per
  * block, blocks per SM the plan is sized for, epilogue warps, 128-row tiles
  * per group, shared-memory bytes per block, tensor-memory columns per block,
- * grid size, form (0: one MMA per 3x3 tap and 128-row tile of padded
- * positions; 1: the local energy's row form, rows = (lattice row,
- * configuration) and x positions along tensor-memory columns). Returns NQS_ERR_INVALID_ARG for a bad problem or argument,
+ * grid size (local energies: of one block per sample; a call that leaves
+ * half of those blocks idle may launch two, four or eight per sample), form
+ * (0: one MMA per 3x3 tap and 128-row tile of padded positions; 1: either of
+ * the local energy's row forms, rows = (lattice row, configuration) and x
+ * positions along tensor-memory columns; nqs_tc_form tells them apart).
+ * Returns NQS_ERR_INVALID_ARG for a bad problem or argument,
  * NQS_ERR_UNSUPPORTED if the tensor-core path cannot run p (channels other
  * than 16 or 32, or no plan fits). */
 int nqs_tc_plan(const nqs_problem *p, int32_t kind, int64_t n, int32_t max_smem_per_block, int32_t num_sms,
                 int32_t *out);
+
+/* The form of that plan, with the arguments and errors of nqs_tc_plan (host
+ * only): 0 = tap form, 1 = row form (all MMAs of a layer before its epilogue;
+ * also the form of NQS_FP8), 2 = wide row form (the two halves of a layer's
+ * columns overlapped with the epilogue); a negative nqs_status on error. */
+int nqs_tc_form(const nqs_problem *p, int32_t kind, int64_t n, int32_t max_smem_per_block, int32_t num_sms);
 
 /* Create a context on the current CUDA device.
  * params: device float64 [nqs_param_count(p)], caller-owned and borrowed

@@ -164,6 +164,16 @@ int check_ctx(nqs_ctx *c) {
     return NQS_OK;
 }
 
+// Both plan queries: form as TcPlan::rows.
+int tc_plan_query(const nqs_problem *q, int32_t kind, int64_t n, int32_t max_smem_per_block, int32_t num_sms,
+                  int32_t *out, int *form) {
+    std::string why;
+    if (!out || kind < 0 || kind > 2 || n < 1 || max_smem_per_block <= 0 || num_sms <= 0) return NQS_ERR_INVALID_ARG;
+    if (!valid_problem(q, &why)) return NQS_ERR_INVALID_ARG;
+    if (kind == 2 && n > INT32_MAX) return NQS_ERR_INVALID_ARG;
+    return tc_describe_plan(make_problem(q), kind, n, (size_t)max_smem_per_block, num_sms, out, form, &why);
+}
+
 }  // namespace
 
 extern "C" {
@@ -176,11 +186,15 @@ int64_t nqs_param_count(const nqs_problem *q) {
 
 int nqs_tc_plan(const nqs_problem *q, int32_t kind, int64_t n, int32_t max_smem_per_block, int32_t num_sms,
                 int32_t *out) {
-    std::string why;
-    if (!out || kind < 0 || kind > 2 || n < 1 || max_smem_per_block <= 0 || num_sms <= 0) return NQS_ERR_INVALID_ARG;
-    if (!valid_problem(q, &why)) return NQS_ERR_INVALID_ARG;
-    if (kind == 2 && n > INT32_MAX) return NQS_ERR_INVALID_ARG;
-    return tc_describe_plan(make_problem(q), kind, n, (size_t)max_smem_per_block, num_sms, out, &why);
+    int form;
+    return tc_plan_query(q, kind, n, max_smem_per_block, num_sms, out, &form);
+}
+
+int nqs_tc_form(const nqs_problem *q, int32_t kind, int64_t n, int32_t max_smem_per_block, int32_t num_sms) {
+    int32_t out[9];
+    int form = 0;
+    const int rc = tc_plan_query(q, kind, n, max_smem_per_block, num_sms, out, &form);
+    return rc == NQS_OK ? form : rc;
 }
 
 int nqs_init(nqs_ctx **out, const nqs_problem *q, double *params, uint64_t seed, void *stream) {

@@ -112,9 +112,9 @@ int launch_wait_probe(int64_t iterations, const LaunchEnv &env);
 int launch_bounds_probe(const LaunchEnv &env);
 // Tensor-core plan the launchers choose (host only): kind 0 log psi, 1 local
 // energy, 2 sampler (n = chains). out[9]: G, slots, blocks per SM, epilogue
-// warps, tiles per group, shared bytes per block, TMEM columns, grid, form
-// (0 tap form, 1 row form).
-int tc_describe_plan(const Problem &p, int kind, int64_t n, size_t max_smem, int num_sms, int32_t *out,
+// warps, tiles per group, shared bytes per block, TMEM columns, grid, 1 for
+// either row form; *form: 0 tap form, 1 row form, 2 wide row form.
+int tc_describe_plan(const Problem &p, int kind, int64_t n, size_t max_smem, int num_sms, int32_t *out, int *form,
                      std::string *why);
 int launch_sample_tc(const Problem &p, const double *p64, const void *packed, int8_t *chains, int n_chains,
                      uint64_t step0, uint64_t seed, int spc, int sweeps_between, int burn_in, int8_t *out_cfg,

@@ -3371,7 +3371,7 @@ int launch_wait_probe(int64_t iterations, const LaunchEnv &env) {
     return check(env, "wait_probe_kernel");
 }
 
-int tc_describe_plan(const Problem &p, int kind, int64_t n, size_t max_smem, int num_sms, int32_t *out,
+int tc_describe_plan(const Problem &p, int kind, int64_t n, size_t max_smem, int num_sms, int32_t *out, int *form,
                      std::string *why) {
     TcPlan pl;
     int per_block = 1;
@@ -3397,6 +3397,7 @@ int tc_describe_plan(const Problem &p, int kind, int64_t n, size_t max_smem, int
     out[6] = (int32_t)pl.tmem_cols;
     out[7] = (int32_t)grid;
     out[8] = pl.rows != 0;
+    *form = pl.rows;
     return NQS_OK;
 }
 

@@ -28,7 +28,7 @@ EXPORTS = ('nqs_param_count', 'nqs_init', 'nqs_destroy', 'nqs_last_error', 'nqs_
            'nqs_logpsi',
            'nqs_connected', 'nqs_local_energy', 'nqs_local_energy_multi', 'nqs_sample', 'nqs_get_chains', 'nqs_set_chains',
            'nqs_logpsi_grad', 'nqs_logpsi_vjp', 'nqs_logpsi_grad_noalloc', 'nqs_noalloc_last_error', 'nqs_sr_solve',
-           'nqs_sr_solve_woodbury', 'nqs_set_sx_arithmetic', 'nqs_tc_plan', 'nqs_probe_wait_timeout', 'nqs_probe_bounds', 'nqs_set_sm_limit',
+           'nqs_sr_solve_woodbury', 'nqs_set_sx_arithmetic', 'nqs_tc_plan', 'nqs_tc_form', 'nqs_probe_wait_timeout', 'nqs_probe_bounds', 'nqs_set_sm_limit',
            'nqs_sampler_counts')
 
 
@@ -63,6 +63,7 @@ def load(path=None):
     sig = {
         'nqs_param_count': (I64, [ctypes.POINTER(nqs_problem)]),
         'nqs_tc_plan': (ctypes.c_int, [ctypes.POINTER(nqs_problem), I32, I64, I32, I32, ctypes.POINTER(I32)]),
+        'nqs_tc_form': (ctypes.c_int, [ctypes.POINTER(nqs_problem), I32, I64, I32, I32]),
         'nqs_init': (ctypes.c_int, [ctypes.POINTER(P), ctypes.POINTER(nqs_problem), P, U64, P]),
         'nqs_destroy': (ctypes.c_int, [P]),
         'nqs_last_error': (ctypes.c_char_p, [P]),
@@ -134,21 +135,23 @@ def nqs_param_count(problem):
 TC_PLAN_KIND = {'logpsi': 0, 'local_energy': 1, 'sample': 2}
 TC_PLAN_FIELDS = ('G', 'slots', 'blocks_per_sm', 'epilogue_warps', 'tiles', 'smem_bytes', 'tmem_cols', 'grid',
                   'row_form')
+TC_FORMS = ('tap', 'row', 'wide')
 
 
 def tc_plan(problem, kind, n, max_smem_per_block=232448, num_sms=152):
     """nqs_tc_plan: the tensor-core plan the launchers choose (host only).
     kind: 'logpsi', 'local_energy' (n = samples) or 'sample' (n = chains).
-    Returns a dict of TC_PLAN_FIELDS, or None if the tensor-core path cannot
+    Returns a dict of TC_PLAN_FIELDS and 'form' (nqs_tc_form: one of TC_FORMS;
+    row_form is 1 for 'row' and 'wide'), or None if the tensor-core path cannot
     run the problem."""
     out = (ctypes.c_int32 * 9)()
-    rc = load().nqs_tc_plan(ctypes.byref(problem), TC_PLAN_KIND[kind], int(n), int(max_smem_per_block), int(num_sms),
-                            out)
+    args = (ctypes.byref(problem), TC_PLAN_KIND[kind], int(n), int(max_smem_per_block), int(num_sms))
+    rc = load().nqs_tc_plan(*args, out)
     if rc == NQS_ERR_UNSUPPORTED:
         return None
     if rc != 0:
         raise NQSError(rc, 'nqs_tc_plan: invalid argument')
-    return dict(zip(TC_PLAN_FIELDS, list(out)))
+    return dict(zip(TC_PLAN_FIELDS, list(out)), form=TC_FORMS[load().nqs_tc_form(*args)])
 
 
 def local_energy_multi(contexts, configs, precision='bf16', outs=None, logpsi=None, max_blocks=0):

@@ -173,6 +173,38 @@ def test_local_energy_row_form_equals_tap_form(case, give_logpsi, monkeypatch):
     assert abs(got[:, 0].mean() - want.real.mean()) / L ** 2 <= 1e-4
 
 
+PLAIN_ROW_CASES = [
+    ('j1j2_10x10', {'n_layers': 1}),
+    ('j1j2_10x10', {'n_layers': 2}),
+    ('j1j2_10x10', {'L': 8, 'n_up': 32, 'n_down': 32, 'n_layers': 2}),
+    ('j1j2_10x10', {'L': 13, 'n_up': 85, 'n_down': 84, 'n_layers': 2}),
+    ('j1j2_10x10', {'L': 6, 'n_up': 18, 'n_down': 18, 'n_layers': 3}),
+    ('tj_12x12', {'L': 7, 'n_up': 22, 'n_down': 22, 'channels': 16, 'n_layers': 3}),
+    ('tj_12x12', {'L': 5, 'n_up': 11, 'n_down': 11, 'channels': 16, 'n_layers': 1}),
+    ('j1j2_10x10', {'L': 4, 'n_up': 8, 'n_down': 8, 'channels': 32, 'n_layers': 4}),
+    ('j1j2_10x10', {'L': 5, 'n_up': 13, 'n_down': 12, 'channels': 32, 'n_layers': 3}),
+    ('tj_12x12', {'L': 4, 'n_up': 6, 'n_down': 6, 'n_layers': 2}),
+]
+
+
+@pytest.mark.parametrize('case', PLAIN_ROW_CASES, ids=_ids)
+def test_local_energy_plain_row_form_equals_tap_form(case, monkeypatch):
+    """The row form that is not the wide one, on what still runs in it (few layers, small lattices with 32 channels):
+    bitwise the tap form, with log psi recomputed and supplied."""
+    from tests.gpu_common import problem_of
+    name, over = case
+    w = WL[name]
+    assert lib().tc_plan(problem_of(w, **over), 'local_energy', 4096)['form'] == 'row'
+    ctx, _ = make_ctx(w, **over)
+    cfg = dev(configs_for(w, 37, seed=49, **over))
+    lp = ctx.logpsi(cfg, 'bf16')
+    rows = ctx.local_energy(cfg, None, 'bf16'), ctx.local_energy(cfg, lp, 'bf16')
+    monkeypatch.setenv('NQS_TC_ROWS', '0')
+    tap = ctx.local_energy(cfg, None, 'bf16'), ctx.local_energy(cfg, lp, 'bf16')
+    ctx.sync()
+    assert torch.equal(rows[0], tap[0]) and torch.equal(rows[1], tap[1])
+
+
 WIDE_CASES = [
     ('j1j2_16x16', {'n_layers': 4}),
     ('j1j2_16x16', {'L': 15, 'n_up': 113, 'n_down': 112, 'n_layers': 7}),

@@ -126,3 +126,26 @@ def test_unsupported_and_invalid(nqs):
         nqs.tc_plan(bad, 'local_energy', 8)
     with pytest.raises(nqs.NQSError):
         nqs.tc_plan(nqs.make_problem('j1j2', 4, n_layers=2, channels=16), 'local_energy', 0)
+
+
+@pytest.mark.parametrize('model,L,channels,layers,form', [
+    ('j1j2', 10, 16, 6, 'wide'), ('j1j2', 10, 16, 3, 'wide'), ('j1j2', 10, 16, 2, 'row'), ('j1j2', 8, 16, 1, 'row'),
+    ('j1j2', 6, 16, 4, 'wide'), ('j1j2', 6, 16, 3, 'row'), ('j1j2', 14, 16, 6, 'tap'), ('tj', 7, 16, 3, 'row'),
+    ('tj', 8, 16, 6, 'tap'), ('j1j2', 4, 32, 6, 'row'), ('j1j2', 5, 32, 2, 'row'), ('j1j2', 6, 32, 1, 'wide'),
+    ('j1j2', 16, 32, 8, 'wide'), ('j1j2', 20, 32, 4, 'tap')])
+def test_form_of_the_local_energies(nqs, model, L, channels, layers, form):
+    """The plan names the form that the launcher takes: tap, row or wide row form (row_form covers the last two)."""
+    N = L * L
+    n = N if model == 'j1j2' else N - N // 8
+    plan = nqs.tc_plan(nqs.make_problem(model, L, n_up=n // 2, n_down=n - n // 2, n_layers=layers, channels=channels),
+                       'local_energy', 4096, MAX_SMEM, NUM_SMS)
+    assert plan['form'] == form and plan['row_form'] == (form != 'tap')
+
+
+def test_form_of_the_other_calls_and_errors(nqs):
+    p = nqs.make_problem('j1j2', 10, n_layers=6, channels=16)
+    assert nqs.tc_plan(p, 'logpsi', 4096)['form'] == 'tap' and nqs.tc_plan(p, 'sample', 256)['form'] == 'tap'
+    form = nqs.load().nqs_tc_form
+    bad = nqs.make_problem('j1j2', 4, n_up=3, n_down=3, n_layers=2, channels=16)
+    assert form(bad, 1, 8, MAX_SMEM, NUM_SMS) == -1 and form(p, 3, 8, MAX_SMEM, NUM_SMS) == -1
+    assert form(nqs.make_problem('j1j2', 4, n_layers=2, channels=4), 1, 8, MAX_SMEM, NUM_SMS) == -7
