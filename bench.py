@@ -626,7 +626,7 @@ def eloc_algorithmic_flops(w, n_samples, pairs, n_conn):
     return float(cone), float((n_samples + n_nn + n_nnn) * dense)
 
 
-TRAFFIC_SOURCES = ('tc.cu', 'tc_ptx.cuh', 'common.cuh', 'internal.h')
+TRAFFIC_SOURCES = ('tc.cu', 'tc_ptx.cuh', 'wide_list.cuh', 'common.cuh', 'internal.h')
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one E_loc launch captured by ncu under
 # `bench.py --profile-eloc 2048`, with the hash of the kernel sources it was taken on
 TRAFFIC_RECORD = {'kernel': 'eloc_wide_kernel', 'samples': 2048, 'dram_bytes': 328960,

@@ -40,6 +40,7 @@
 
 #include "internal.h"
 #include "tc_ptx.cuh"
+#include "wide_list.cuh"
 
 namespace nqs {
 
@@ -1168,12 +1169,6 @@ __device__ __forceinline__ WideRow wide_row(const TcPlan &pl, const TcShared &sh
     return r;
 }
 
-// One configuration of the group: sigma with sites i and j exchanged (-1: as
-// it is), rolled along x: its column c is sigma's column c + roll.
-struct WideCfg {
-    int16_t i, j, roll, pad;
-};
-
 // The group's configurations: entries first .. first + count - 1 of the
 // connected list in evaluation order (negative: the sample itself; slots past
 // count repeat it). cfgs holds them for groups with a class (their rolls).
@@ -1181,11 +1176,12 @@ struct WideEntries {
     const int16_t *ci, *cj, *ord;
     const WideCfg *cfgs;
     int first, count, cls;
+    int nconn, N;   // list entries and sites, for the checked build
+    int *err;
     __device__ __forceinline__ WideCfg get(int g) const {
         if (cls >= 0) return cfgs[g];
         if (g >= count || first + g < 0) return WideCfg{-1, -1, 0, 0};
-        const int k = ord[first + g];
-        return WideCfg{ci[k], cj[k], 0, 0};
+        return wide_entry(ci, cj, ord[first + g], nconn, N, err);
     }
     __device__ __forceinline__ int roll(int g) const { return cls < 0 ? 0 : cfgs[g].roll; }
 };
@@ -1618,16 +1614,14 @@ __device__ bool wide_sample(const TcPlan &pl, const Problem &p, TcShared &sh, Tc
             // the group's class is its last entry's (class 1's band covers class 0); dense if it holds the sample
             int cls = -1;
             if (cone && e0 >= lead + first) {
-                const int k = e.ord[e0 + cnt - 1 - lead];
-                cls = e.ci[k] % L != e.cj[k] % L;
+                const WideCfg v = wide_entry(e.ci, e.cj, e.ord[e0 + cnt - 1 - lead], nconn, N, err);
+                cls = v.i % L != v.j % L;
             }
             if (cls >= 0) {
                 if (threadIdx.x < G) {
                     WideCfg v{-1, -1, 0, 0};
                     if ((int)threadIdx.x < cnt) {
-                        const int k = e.ord[e0 + threadIdx.x - lead];
-                        v.i = e.ci[k];
-                        v.j = e.cj[k];
+                        v = wide_entry(e.ci, e.cj, e.ord[e0 + threadIdx.x - lead], nconn, N, err);
                         const int r = v.i % L - (L / 2 - 1);   // the bond's first site is the left one: to column H - 1
                         v.roll = (int16_t)(r < 0 ? r + L : r);
                     }
@@ -1635,12 +1629,13 @@ __device__ bool wide_sample(const TcPlan &pl, const Problem &p, TcShared &sh, Tc
                 }
                 __syncthreads();
             }
-            const WideEntries ent{e.ci, e.cj, e.ord, e.cfgs, e0 - lead, cnt, cls};
+            const WideEntries ent{e.ci, e.cj, e.ord, e.cfgs, e0 - lead, cnt, cls, nconn, N, err};
             ok = wide_forward<C>(pl, sh, packed, st, err, e.sigma, ent, cache, cone && lead && e0 == 0 ? cache : nullptr);
             if (ok && threadIdx.x < cnt) {
                 const int q = e0 + (int)threadIdx.x - lead, idx = q < 0 ? 0 : e.ord[q] + lead;
                 const float la = (float)sh.res[threadIdx.x], lphi = (float)sh.res[G + threadIdx.x];
-                if (rank != 0) {
+                if (!NQS_INDEX_OK(idx >= 0 && idx < n_entries, err)) {   // this block's list or block 0's
+                } else if (rank != 0) {
                     ptx::st_cluster_v2f32(ptx::smem_u32(e.lp + 2 * idx), 0, la, lphi);
                 } else {
                     e.lp[2 * idx] = la;
