@@ -1081,9 +1081,12 @@ __host__ __device__ inline size_t wide_cache_bytes(const TcPlan &pl) {
 // halves innermost. Broadcast values and the split into edge and interior
 // columns keep the descriptors in uniform registers with two additions an
 // interior MMA, so that one thread issues as fast as the operand path takes
-// them (45 cycles at N = 48, 54 at N = 96 on an idle SM; 66 and 57 with the
-// columns in one loop; the election in every MMA cost 8 - 17 % of the whole
-// kernel). All of that is computed before the wait for the stage: it stood
+// them: 44.1 cycles an MMA at N = 48 and 56.1 at N = 96 back to back (operand
+// bytes over 128 B a clock: 44, 56), and over a layer's MMAs of all widths
+// 42.1 at 10 x 10 x 16 channels and 52.5 at 16 x 16 x 32 (operands 41.9, 51.9;
+// 50.3 and 55.0 for one layer by itself with the latency at its end). With the
+// columns in one loop a layer took 21 and 3 cycles an MMA more; the election in
+// every MMA cost 8 - 17 % of the whole kernel. All of that is computed before the wait for the stage: it stood
 // between the stage and the first MMA, ~500 cycles a layer (11.02 -> 10.85 ms
 // for 8,192 samples at 10 x 10 x 16 channels, 67.8 -> 64.9 ms for 4,096 at
 // 16 x 16 x 32). False if a wait gave up.
