@@ -2104,33 +2104,61 @@ struct TcRequest {
 // the single-problem kernel: descriptors stay in uniform registers). Blocks
 // take samples one at a time from a global counter in problem-major order and
 // re-bind their shared-memory plan when the problem changes. Dense: cones pay
-// only on the largest lattices. Requests of one shape share a plan, so that
-// the 32,764 bytes of a kernel's parameters hold more requests than there are
-// SMs: a launch of fewer would leave SMs idle that one launch of every request
-// keeps busy (32 channels, six layers, one to four samples a request, ms for 33
-// / 120 / 250 requests of 10x10 and 12x12: 2.19 / 7.17 / 14.7 in launches of 16,
-// 0.98 / 2.14 / 4.92 here, 1.71 / 3.68 / 7.51 in one tap-form launch).
-constexpr int kWideGroupPlans = 24;
-constexpr int kWideGroupMax = 220;
-struct WideRequest {
-    Problem p;
-    const unsigned char *packed;
-    const int8_t *configs;
-    const double *logpsi;
-    double *out;
-    int64_t start;   // index of the request's first sample in the launch
-    int plan;
-};
-struct WideGroup {
-    int count, plans;
-    TcPlan pl[kWideGroupPlans];
-    WideRequest r[kWideGroupMax];
-};
-static_assert(sizeof(WideGroup) + 64 <= 32764, "the requests are kernel parameters");
+// only on the largest lattices. Past 16 requests those of one shape share a
+// plan, so that the 32,764 bytes of a kernel's parameters hold more requests
+// than there are SMs: a launch of fewer would leave SMs idle that one launch of
+// every request keeps busy (32 channels, six layers, one to four samples a
+// request, ms for 33 / 120 / 250 requests of 10x10 and 12x12: 2.19 / 7.17 /
+// 14.7 in launches of 16, 0.98 / 2.14 / 4.92 here, 1.71 / 3.68 / 7.51 in one
+// tap-form launch). A shared plan costs a smaller group 0.2 % and its larger
+// parameters 2 us.
+struct WideGroupSmall {
+    static constexpr int kMost = 16;
+    int count;
+    TcRequest r[kMost];
 
-template <int C>
+    __device__ __forceinline__ const TcPlan &plan(const TcRequest &q) const { return q.pl; }
+    // Append request q with plan pl, its samples from start on; false if the group is full.
+    bool add(const TcRequest &q, const TcPlan &pl, int64_t start) {
+        if (count == kMost) return false;
+        r[count] = q;
+        r[count].pl = pl;
+        r[count++].start = start;
+        return true;
+    }
+};
+
+struct WideGroupLarge {
+    static constexpr int kMost = 220, kPlans = 24;
+    struct Request {
+        Problem p;
+        const unsigned char *packed;
+        const int8_t *configs;
+        const double *logpsi;
+        double *out;
+        int64_t start;   // index of the request's first sample in the launch
+        int plan;
+    };
+    int count, plans;
+    TcPlan pl[kPlans];
+    Request r[kMost];
+
+    // the index in a register: read at every use of the plan it cost 5 - 9 %
+    __device__ __forceinline__ const TcPlan &plan(const Request &q) const { return pl[__shfl_sync(0xffffffffu, q.plan, 0)]; }
+    bool add(const TcRequest &q, const TcPlan &with, int64_t start) {
+        int k = 0;
+        while (k < plans && std::memcmp(&pl[k], &with, sizeof(TcPlan)) != 0) ++k;
+        if (k == kPlans || count == kMost) return false;
+        if (k == plans) pl[plans++] = with;
+        r[count++] = Request{q.p, q.packed, q.configs, q.logpsi, q.out, start, k};
+        return true;
+    }
+};
+static_assert(sizeof(WideGroupLarge) + 64 <= 32764, "the requests are kernel parameters");
+
+template <int C, typename Group>
 __global__ void __launch_bounds__(kWideThreads<C>, kWideBlocks<C>)
-    eloc_wide_multi_kernel(const __grid_constant__ WideGroup grp, int64_t total, uint32_t tmem_cols,
+    eloc_wide_multi_kernel(const __grid_constant__ Group grp, int64_t total, uint32_t tmem_cols,
                            unsigned long long *counter, int *err) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ long long grab;
@@ -2150,8 +2178,8 @@ __global__ void __launch_bounds__(kWideThreads<C>, kWideBlocks<C>)
             if (grp.r[mid].start <= g) r = mid;
             else end = mid;
         }
-        const WideRequest &q = grp.r[r];
-        const TcPlan &pl = grp.pl[__shfl_sync(0xffffffffu, q.plan, 0)];   // the index in a register, not read at every use
+        const auto &q = grp.r[r];
+        const TcPlan &pl = grp.plan(q);
         if (r != cur) {
             if (cur >= 0) tc_unbind(sh, st);
             row_bind(pl, sh, q.packed, st);
@@ -3136,7 +3164,7 @@ int launch_eloc_tc(const Problem &p, const double *, const void *packed, const i
 size_t tc_multi_table_bytes(int count) { return 256 + sizeof(TcRequest) * (size_t)count; }
 
 // Each problem runs in the form its own launch would choose: those with a wide
-// plan in launches of up to kWideGroupMax problems, the others in one tap-form
+// plan in launches of WideGroupSmall or WideGroupLarge, the others in one tap-form
 // launch. A mix of six requests (J1-J2 6x6 .. 12x12, t-J 6x6 and 12x12, both
 // channel counts, 4 layers, 512 - 2,048 samples): 11.8 ms with every problem in
 // the tap form at one block per SM, 6.2 ms this way. The launches follow each
@@ -3214,30 +3242,28 @@ int launch_eloc_tc_multi(const TcMultiItem *items, int count, void *dev_table, i
     // max_blocks is a share in SMs: the blocks that fill one SM count as one (16 channels, 1,536 samples of 10x10 to
     // 6x6 capped at all 152 SMs: 1.64 ms with 152 half-SM blocks, 1.01 with 304)
     const auto grid_of = [&](int64_t total, int ctas) { return (int)std::max<int64_t>(1, std::min(total, slots * ctas)); };
-    for (size_t w0 = 0; w0 < wide.size();) {
-        WideGroup grp{};
+    size_t w0 = 0;
+    auto launch_wide = [&](auto grp) -> int {   // the next requests, as many as grp holds
         uint32_t smem = 0, cols = 32;
         int64_t total = 0;
-        for (; w0 < wide.size() && grp.count < kWideGroupMax; ++w0, ++grp.count) {
-            const Member &m = *wide[w0];
-            int k = 0;
-            while (k < grp.plans && std::memcmp(&grp.pl[k], &m.wide, sizeof(TcPlan)) != 0) ++k;
-            if (k == kWideGroupPlans) break;
-            if (k == grp.plans) grp.pl[grp.plans++] = m.wide;
-            grp.r[grp.count] = WideRequest{m.r.p, m.r.packed, m.r.configs, m.r.logpsi, m.r.out, total, k};
-            total += m.r.n;
-            smem = std::max(smem, m.wide.total);   // each plan already keeps to its blocks per SM
-            cols = std::max(cols, m.wide.tmem_cols);
+        const TcPlan &first = wide[w0]->wide;
+        for (; w0 < wide.size() && grp.add(wide[w0]->r, wide[w0]->wide, total); ++w0) {
+            total += wide[w0]->r.n;
+            smem = std::max(smem, wide[w0]->wide.total);   // each plan already keeps to its blocks per SM
+            cols = std::max(cols, wide[w0]->wide.tmem_cols);
         }
         if (int rc = reset()) return rc;
-        const int grid = grid_of(total, grp.pl[0].ctas), threads = 32 * (grp.pl[0].epi + kIssuers);
+        const int grid = grid_of(total, first.ctas), threads = 32 * (first.epi + kIssuers);
         NQS_TC_DISPATCH(C, {
-            auto k = eloc_wide_multi_kernel<CC>;
+            auto k = eloc_wide_multi_kernel<CC, decltype(grp)>;
             if (int rc = allow_dynamic_smem(k, smem, env)) return rc;
             k<<<grid, threads, smem, env.stream>>>(grp, total, cols, counter, env.err);
         });
-        if (int rc = check(env, "eloc_wide_multi_kernel")) return rc;
-    }
+        return check(env, "eloc_wide_multi_kernel");
+    };
+    while (w0 < wide.size())
+        if (int rc = wide.size() - w0 <= WideGroupSmall::kMost ? launch_wide(WideGroupSmall{}) : launch_wide(WideGroupLarge{}))
+            return rc;
     if (tap.empty()) return NQS_OK;
     uint32_t smem = 0, cols = 32;
     int64_t total = 0;
