@@ -2256,8 +2256,8 @@ __device__ __forceinline__ int neighbour_dir_tc(int i, int d, int L) {
 // 1.20, 1.68 / 1.34, 1.63 / 1.48; 1,024 chains 4.86 / 3.31, 4.84 / 3.62, 4.68 /
 // 4.15. t-J 12x12, 32 channels, 256 chains, 0.53: 6.10 / 5.07. 16x16, 32
 // channels, 8 layers, 128 chains: 12.6 / 5.6.
-// `typical` starts anew in every launch and its first steps are long: a launch
-// of one sweep whose moves are almost all rejected otherwise ends before the
+// `typical` starts anew in every launch, with long first steps: a launch of one
+// sweep whose moves are almost all rejected otherwise ends before the
 // prediction has found them (us, one sweep of 64 chains with an acceptance of
 // 0.02, one proposal at a time / steps of at most 0.05 / these steps: 10x10, 32
 // channels, 6 layers 487 / 622 / 360; 8x8 340 / 422 / 225; 1,024 chains at
@@ -2267,7 +2267,7 @@ __device__ __forceinline__ int neighbour_dir_tc(int i, int d, int L) {
 template <int C>
 __device__ bool sample_ahead(const TcPlan &pl, const TcShared &sh, const unsigned char *packed, TcState &st, int *err,
                              int8_t *cur, int *wpi, int *wpj, double *wlu, int W, int64_t &wbase, float *typical,
-                             float *bias, int *advance, double *ca, double *cphi, unsigned long long *counts, int64_t first,
+                             float *reach, int *advance, double *ca, double *cphi, unsigned long long *counts, int64_t first,
                              int64_t n_steps, uint64_t chain, uint64_t step0, uint64_t seed) {
     const int G = pl.G, N = pl.N, lane = threadIdx.x & 31;
     int q = 0;   // next proposal of the sweep
@@ -2355,15 +2355,10 @@ __device__ bool sample_ahead(const TcPlan &pl, const TcShared &sh, const unsigne
             const uint32_t wrong = (accepted ^ pred) & ((1u << m) - 1u);
             const int last = wrong ? __ffs(wrong) - 1 : m - 1;
             const uint32_t took = accepted & ((2u << last) - 1u);
-            // typical moves to the decided moves' centre: a step of a quarter of each one's distance, which counts for
-            // at most 0.2, or half the average signed distance of late while that is larger
-            const float dist = lane <= last ? (float)delta - *typical : 0.f, cut = fmaxf(0.2f, 0.5f * fabsf(*bias));
-            float pull = fminf(fmaxf(dist, -cut), cut), mean = fminf(fmaxf(dist, -20.f), 20.f);
+            // typical moves by a quarter of each decided move's distance from it, which counts for at most *reach
+            float pull = lane <= last ? fminf(fmaxf((float)delta - *typical, -*reach), *reach) : 0.f;
 #pragma unroll
-            for (int o = 1; o < kMaxAhead; o <<= 1) {
-                pull += __shfl_xor_sync(0xffffffffu, pull, o);
-                mean += __shfl_xor_sync(0xffffffffu, mean, o);
-            }
+            for (int o = 1; o < kMaxAhead; o <<= 1) pull += __shfl_xor_sync(0xffffffffu, pull, o);
             if (lane == 0) {
                 int adv = avail;   // every prediction right, fewer than G moves: none is left among these proposals
 #pragma unroll
@@ -2382,7 +2377,7 @@ __device__ bool sample_ahead(const TcPlan &pl, const TcShared &sh, const unsigne
                 counts[0] += (unsigned long long)(last + 1);
                 counts[1] += (unsigned long long)__popc(took);
                 *typical += 0.25f * pull;
-                *bias += 0.25f * (mean / (float)(last + 1) - *bias);
+                *reach = fmaxf(0.2f, 0.8f * *reach);
                 *advance = adv;
             }
         }
@@ -2454,22 +2449,21 @@ __global__ void __launch_bounds__(kTcThreads, 2) sample_tc_kernel(TcPlan pl, con
     }
     const int n_sweeps = burn_in + spc * sweeps_between;
     const int64_t n_steps = (int64_t)n_sweeps * N;
-    // AHEAD: step of the window's first proposal; in shared memory, 2 (a' - a) of a typical move, the decided moves'
-    // average signed distance from it (16: not known yet, it may take long steps) and the proposals decided by the
-    // last forward
+    // AHEAD: step of the window's first proposal; in shared memory, 2 (a' - a) of a typical move, four times the longest
+    // step that one move may give it (shorter with every forward) and the proposals decided by the last forward
     int64_t wbase = -W;
-    float *typical = reinterpret_cast<float *>(list2), *bias = typical + 1;
+    float *typical = reinterpret_cast<float *>(list2), *reach = typical + 1;
     int *advance = list2 + 2;
     if (AHEAD) {
         if (threadIdx.x == 0) {
             *typical = 0.f;
-            *bias = 16.f;
+            *reach = 16.f;
         }
         __syncthreads();
     }
     for (int sweep = 0; ok && sweep < n_sweeps; ++sweep) {
         if constexpr (AHEAD) {
-            ok = sample_ahead<C>(pl, sh, packed, st, err, cur, wpi, wpj, wlu, W, wbase, typical, bias, advance, ca,
+            ok = sample_ahead<C>(pl, sh, packed, st, err, cur, wpi, wpj, wlu, W, wbase, typical, reach, advance, ca,
                                  cphi, scnt(),
                                  (int64_t)sweep * N, n_steps, (uint64_t)c0, step0, seed);
             if (!ok) break;
