@@ -460,6 +460,10 @@ __global__ void __launch_bounds__(128) vjp_reduce_kernel(const double *__restric
 // holds, counted in rounds of the block's threads (a forward or input-gradient
 // tile is 72 C packed multiply-adds, a weight-gradient tile 9 N R), the
 // cheapest per sample; fewer if the call has fewer samples than SMs times S.
+// Lattices whose two streams do not fit (24x24 and 25x25 with 16 channels,
+// 17x17 with 32) run the backward once a stream, which is still shorter than
+// the kernel before, which carried both (three layers, 400 samples, us: 839 ->
+// 515, 951 -> 550, 1,375 -> 834).
 int grad_streams(const Problem &p, bool vjp, size_t max_smem) {
     return !vjp && grad_layout(p, 1, 2, false).total + 1024 <= max_smem ? 2 : 1;
 }

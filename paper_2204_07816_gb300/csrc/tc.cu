@@ -2251,17 +2251,19 @@ __device__ __forceinline__ int neighbour_dir_tc(int i, int d, int L) {
 // forward of one configuration is a chain of latencies that leaves the SM
 // mostly idle (one tile of MMAs per layer), and further configurations cost
 // little beside it. Measured (GB300, ms for four sweeps, one proposal at a time
-// / ahead): 10x10, 16 channels, 6 layers: 152 chains 1.55 / 0.84 at an
-// acceptance of 1.0, 1.51 / 1.01 at 0.9, 1.49 / 1.16 at 0.13; 256 chains 1.71 /
-// 1.20, 1.68 / 1.34, 1.63 / 1.48; 1,024 chains 4.86 / 3.31, 4.84 / 3.62, 4.68 /
-// 4.15. t-J 12x12, 32 channels, 256 chains, 0.53: 6.10 / 5.07. 16x16, 32
-// channels, 8 layers, 128 chains: 12.6 / 5.6.
+// / ahead): 10x10, 16 channels, 6 layers: 152 chains 1.49 / 0.78 at an
+// acceptance of 1.0, 1.49 / 0.94 at 0.9, 1.46 / 0.78 below 0.01; 256 chains
+// 1.67 / 1.14, 1.66 / 1.27, 1.60 / 1.12; 1,024 chains 4.85 / 3.27, 4.75 / 3.61,
+// 4.53 / 3.11. t-J 12x12, 32 channels, 256 chains, 0.49: 6.01 / 5.02. 16x16, 32
+// channels, 8 layers, 128 chains: 12.5 / 5.5 at 1.0, 13.7 / 6.3 at 0.02. Slower
+// only where a forward of four takes four tiles and half its predictions fail
+// (t-J 10x10, 32 channels, 64 chains, acceptance 0.42, one sweep: 548 / 572 us).
 // `typical` starts anew in every launch, with long first steps: a launch of one
 // sweep whose moves are almost all rejected otherwise ends before the
 // prediction has found them (us, one sweep of 64 chains with an acceptance of
 // 0.02, one proposal at a time / steps of at most 0.05 / these steps: 10x10, 32
-// channels, 6 layers 487 / 622 / 360; 8x8 340 / 422 / 225; 1,024 chains at
-// 6x6, 16 channels, 6 layers 453 / 522 / 312).
+// channels, 6 layers 487 / 622 / 356; 8x8 340 / 422 / 220; 1,024 chains at
+// 6x6, 16 channels, 6 layers 453 / 522 / 305).
 // Every thread follows the state (the last block barrier followed its update)
 // and every warp picks the proposals by itself, its lanes over the next 32.
 template <int C>
@@ -2808,8 +2810,10 @@ bool use_row_form(const Problem &p, size_t max_smem, bool f8, TcPlan *out) {
     // The wide form where it is the faster one (GB300, ms, wide / the other form; 2,432 samples at 16 channels, 1,216
     // at 32). 16 channels, against the row form: from three layers on 8 x 8 and larger and four on smaller lattices
     // (10x10: 1.61 / 1.59 with two layers, 2.49 / 2.68 with four, 4.23 / 4.78 with eight; 6x6: 0.46 / 0.43, 0.68 /
-    // 0.68, 1.12 / 1.17). 32 channels, against the tap form: from 6 x 6 (5x5, four layers 0.51 / 0.49; 6x6 0.72 /
-    // 0.79; 10x10 2.64 / 4.15; 16x16, eight layers, cones in both: 20.1 / 37.6).
+    // 0.68, 1.12 / 1.17); lattices whose row plan does not fit (J1-J2 from 14x14, t-J from 8x8) keep the tap form, also
+    // the few where a wide plan of two blocks an SM would fit, which was not measured. 32 channels, against the tap
+    // form: from 6 x 6 (6x6, four layers 0.72 / 0.79; 10x10 2.64 / 4.15; 16x16, eight layers, cones in both: 20.1 /
+    // 37.6); smaller lattices take the row form (5x5, four layers 0.38, in the wide form 0.51, in the tap form 0.48).
     if (p.C == 16 ? !rows || p.n_layers < (p.L >= 8 ? 3 : 4) : p.L < 6) return rows;
     return make_wide_plan(p, max_smem, out, &why, G) || rows;
 }
@@ -3051,7 +3055,11 @@ size_t tc_eloc_cache_bytes(const Problem &p, size_t max_smem, int num_sms, int64
 // 12x12, 32 channels, 8 samples 0.565 / 0.292 / 0.163 / 0.110; 14x14, 32
 // channels, 8 layers, 8 samples 1.73 / 0.89 / 0.48 / 0.26; 6x6, 16 channels,
 // 4 layers, 8 samples 0.092 / 0.057 / 0.048 / 0.048. NQS_TC_SPLIT=K caps it (1:
-// off).
+// off). Lattices with cones (32 channels from 15x15) are not split: a block
+// needs its own evaluation of the sample for its cache. Dense blocks would be
+// the shorter call there up to half the SMs (16x16, 8 layers, 8 / 37 / 75 / 152
+// samples: 2.40 / 2.47 / 2.55 / 2.55 ms with cones, 0.38 / 1.37 / 1.42 / 2.83
+// dense and split).
 template <typename K>
 int wide_split(K kernel, const Problem &p, const TcPlan &pl, int64_t n, int num_sms, cudaLaunchConfig_t *cfg) {
     const char *e = getenv("NQS_TC_SPLIT");
